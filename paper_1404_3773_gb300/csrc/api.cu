@@ -526,6 +526,7 @@ cs_status rr_core(cs_ctx* c, int n_s, double* X, long long ld, double* theta, do
   if (r != CS_OK) return r;
   void* oz = work + lay.oz;
   CS_LAUNCH(c, 2, dense_gram(c, X, ld, HX, H.d, H.d, n_s, n_s, Hs, n_s, part, st, oz));
+  CS_LAUNCH(c, 1, launch_symmetrize(Hs, n_s, st));
   // with slice-product dense steps the eigensolver's refinement products may use them too
   // (the workspace slot holds at least the d x n_s products' split operands)
   const bool sl = c->dense_prec == CS_FP64_SLICED;

@@ -155,6 +155,8 @@ cudaError_t launch_scale_rows(F* y, int n_p, int S, int ld, const F* h, cudaStre
 // work: n*n + 2n doubles. status[0] = 0 ok, else 1 + index of the failing pivot.
 cudaError_t launch_cholqr_factor(const double* M, int n, double* U, double* work, int* status,
                                  cudaStream_t stream);
+// A (n x n) <- (A + A^T) / 2
+cudaError_t launch_symmetrize(double* A, int n, cudaStream_t stream);
 // Symmetric eigensolve of sym(A) (n x n, lda = n): theta ascending, V (n x n) columns. An FP32
 // solve (Householder tridiagonalisation, then bisection with inverse iteration, or QL where the
 // bisection tiles do not fit in shared memory), Newton-Schulz re-orthonormalisation and
