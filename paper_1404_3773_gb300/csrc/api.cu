@@ -25,11 +25,13 @@ thread_local std::string g_init_error;
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Layout {
-  size_t G, Yalt, X32, Wkb, kbZ, HX, tmp, part, small, lanV, status, HXr, chw, oz, wd, kbtc, wa,
+  size_t G, Yalt, X32, Wkb, kbZ, HX, tmp, part, small, lanV, status, HXr, chw, oz, wd, sl, kbtc, wa,
       total;
 };
 
 constexpr int kMaxLanczos = 64;
+// largest block whose eigensolve starts with the one-CTA FP32 stage (launch_sym_eig)
+constexpr int kOneCtaEig = 112;
 // largest degree of the residual-form filter (its weight table is sized for it)
 constexpr int kMaxRitzDegree = 64;
 
@@ -79,6 +81,8 @@ Layout layout(const cs_ctx* c, int n_s, cs_precision prec) {
   o.wd = take(angular_wide_df_eligible(T.L, T.n_theta, T.n_phi)
                   ? angular_wide_df_work_bytes(T.L, T.n_r, T.n_theta)
                   : 0);
+  // intermediates of the slice-product FP64 H.X (one chunk of radial nodes)
+  o.sl = take(c->sliced_ok ? sliced_hx_work_bytes(T.L, T.n_r, T.n_theta, T.n_phi, n_s) : 0);
   // last, so that every other offset is the same for both precisions
   auto is_f32 = [](cs_precision p) { return p == CS_FP32 || p == CS_MIXED_BF16; };
   const bool reduced = is_f32(prec) || is_f32(c->rr_prec);
@@ -228,13 +232,29 @@ cs_status upload_tables(cs_ctx* c) {
   return CS_OK;
 }
 
+// Whether an FP64 (or, with df, a double-float) H.X of n_s states takes the slice products
+// (sliced_hx.cu), by the number of grid rows x states.
+// FP64: they are faster at every size measured (lmax 6 .. 60, 1 .. 130 states): 0.074 against
+// 0.092 ms at 3456 rows, where launches dominate, 0.084 against 0.134 at 5120, 1.50 against 7.13
+// at 460800 (lmax 30, 80 states). Below 4096 rows, with little to gain, the kernels that
+// cs_apply_H_noalloc runs stay.
+// Double-float: its kernels cost less per row at small lmax. rows L^2 = 14M is where the two
+// meet: 0.130 / 0.122 ms at 7.4M (lmax 16, 16 states), 0.177 / 0.181 at 15M (lmax 23, 8),
+// 0.168 / 0.193 at 15M (lmax 16, 32), 0.254 / 0.336 at 44M (lmax 30, 8).
+bool use_sliced(const cs_ctx* c, int n_s, bool df) {
+  if (!c->sliced_ok || !sliced_hx_enabled()) return false;
+  const HostTables& H = c->host;
+  const long long rows = (long long)H.n_r * H.n_theta * n_s;
+  return rows * H.L * H.L >= 14000000 || (!df && rows >= 4096);
+}
+
 // ------------------------------------------------------------------ H.X core
 // out = epilogue(1/2 Lambda X + Z (+ kb)); see Epilogue in hx_kernels.cuh
 template <typename T>
 cs_status hx_core(cs_ctx* c, int n_s, const T* X, long long ldx, T* out, long long ldo, int mode,
                   double cA, double cB, double csh, const T* Yprev, char* work, cudaStream_t st,
                   bool tc = false, const T* src = nullptr, const T* src_w = nullptr,
-                  const T* kb_in = nullptr) {
+                  const T* kb_in = nullptr, bool as_df = false, bool fma = false) {
   const HostTables& H = c->host;
   DevTables<T>& D = tables<T>(c);
   const Layout lay = layout(c, n_s, CS_FP64);
@@ -280,6 +300,35 @@ cs_status hx_core(cs_ctx* c, int n_s, const T* X, long long ldx, T* out, long lo
     }
     kb = kbZ;
   }
+  Epilogue<T> ep;
+  ep.mode = mode;
+  ep.out = out;
+  ep.X = X;
+  ep.ld = ldx;
+  ep.ld_out = ldo;
+  ep.Yprev = Yprev;
+  ep.half_lambda = D.half_lambda;
+  ep.kb = kb;
+  ep.kb_ld = H.d;
+  ep.cA = (T)cA;
+  ep.cB = (T)cB;
+  ep.cshift = (T)csh;
+  ep.src = src;
+  ep.src_w = src_w;
+  ep.src_ld = H.d;
+  if constexpr (std::is_same<T, double>::value) {
+    if (!fma && use_sliced(c, n_s, as_df)) {
+      // as_df: launches of a double-float call, which takes the same products
+      const int base = as_df ? prof_cls<df64>(0) : prof_cls<T>(0);
+      for (int stage = 0; stage < 3; ++stage) {
+        int nl = 0;
+        CS_LAUNCH_CLS(c, base + stage, nl,
+                      launch_sliced_hx(H, c->sliced, n_s, X, ldx, G, ep, work + lay.sl, c->dev_err,
+                                       st, stage, &nl));
+      }
+      return CS_OK;
+    }
+  }
   TcTables tt;
   tt.synth = c->tc_synth;
   tt.anal = c->tc_anal;
@@ -324,22 +373,6 @@ cs_status hx_core(cs_ctx* c, int n_s, const T* X, long long ldx, T* out, long lo
   }
   if (!ang_done)
     CS_LAUNCH_CLS(c, prof_cls<T>(1), 1, launch_angular<T>(a, ANG_FULL, G, nullptr, nullptr, st));
-  Epilogue<T> ep;
-  ep.mode = mode;
-  ep.out = out;
-  ep.X = X;
-  ep.ld = ldx;
-  ep.ld_out = ldo;
-  ep.Yprev = Yprev;
-  ep.half_lambda = D.half_lambda;
-  ep.kb = kb;
-  ep.kb_ld = H.d;
-  ep.cA = (T)cA;
-  ep.cB = (T)cB;
-  ep.cshift = (T)csh;
-  ep.src = src;
-  ep.src_w = src_w;
-  ep.src_ld = H.d;
   if (tc_rad) {
     CS_LAUNCH_CLS(c, prof_cls<T>(2), 1, launch_tc_radial_anal(tt, H, reinterpret_cast<const float*>(G), n_s,
                                                  *reinterpret_cast<const Epilogue<float>*>(&ep),
@@ -355,11 +388,12 @@ cs_status hx_core(cs_ctx* c, int n_s, const T* X, long long ldx, T* out, long lo
 // (only with CS_FP64_SLICED dense products) their term is formed first from the FP64 block as
 // exact slice products, converted to double-float in place and handed to the epilogue.
 cs_status hx_df64_from_fp64(cs_ctx* c, int n_s, const double* X, long long ld, double* HX,
-                            long long ldh, df64* Xd, df64* Yd, char* work, cudaStream_t st);
+                            long long ldh, df64* Xd, df64* Yd, char* work, cudaStream_t st,
+                            bool fma = false);
 
 template <typename T>
 cs_status cheb_core(cs_ctx* c, int n_s, T* X, long long ld, int degree, double a, double b,
-                    double a0, char* work, cudaStream_t st, bool tc = false) {
+                    double a0, char* work, cudaStream_t st, bool tc = false, bool as_df = false) {
   const HostTables& H = c->host;
   const Layout lay = layout(c, n_s, CS_FP64);
   T* alt = reinterpret_cast<T*>(work + lay.Yalt);
@@ -367,7 +401,8 @@ cs_status cheb_core(cs_ctx* c, int n_s, T* X, long long ld, int degree, double a
   const double cc = 0.5 * (a + b), e = 0.5 * (b - a);
   const double s1 = e / (a0 - cc);
   // Y_1 = (sigma_1/e)(H - c) Y_0 into alt
-  cs_status r = hx_core<T>(c, n_s, X, ld, alt, lda, EP_CHEB, s1 / e, 0.0, cc, nullptr, work, st, tc);
+  cs_status r = hx_core<T>(c, n_s, X, ld, alt, lda, EP_CHEB, s1 / e, 0.0, cc, nullptr, work, st, tc,
+                           nullptr, nullptr, nullptr, as_df);
   if (r != CS_OK) return r;
   T* prev = X;
   long long ldp = ld;
@@ -378,7 +413,7 @@ cs_status cheb_core(cs_ctx* c, int n_s, T* X, long long ld, int degree, double a
     double sn = 1.0 / (2.0 / s1 - sig);
     // Y_{i+1} = (2 sn/e)(H - c) Y_i - sig sn Y_{i-1}, written over Y_{i-1}
     r = hx_core<T>(c, n_s, cur, ldc, prev, ldp, EP_CHEB, 2.0 * sn / e, sig * sn, cc, prev, work, st,
-                   tc);
+                   tc, nullptr, nullptr, nullptr, as_df);
     if (r != CS_OK) return r;
     std::swap(prev, cur);
     std::swap(ldp, ldc);
@@ -396,7 +431,8 @@ cs_status cheb_core(cs_ctx* c, int n_s, T* X, long long ld, int degree, double a
 template <typename T>
 cs_status cheb_ritz_core(cs_ctx* c, int n_s, double* X, long long ld, const double* HX,
                          long long ldh, const double* theta, int degree, double a, double b,
-                         double a0, char* work, cudaStream_t st, bool tc = false) {
+                         double a0, char* work, cudaStream_t st, bool tc = false,
+                         bool as_df = false) {
   const HostTables& H = c->host;
   const cs_precision pl = std::is_same<T, float>::value ? (tc ? CS_MIXED_BF16 : CS_FP32) : CS_FP64;
   const Layout lay = layout(c, n_s, pl);
@@ -418,7 +454,8 @@ cs_status cheb_ritz_core(cs_ctx* c, int n_s, double* X, long long ld, const doub
     const double sn = 1.0 / (2.0 / s1 - sig);
     // D_{i+1} = (2 sn/e)[(H - c) D_i + s_i(Theta) R] - sig sn D_{i-1}   (D_0 = 0)
     cs_status r = hx_core<T>(c, n_s, cur, H.d, prev, H.d, EP_CHEB, 2.0 * sn / e, sig * sn, cc,
-                             i == 1 ? nullptr : prev, work, st, tc, R, wt + (size_t)i * n_s);
+                             i == 1 ? nullptr : prev, work, st, tc, R, wt + (size_t)i * n_s, nullptr,
+                             as_df);
     if (r != CS_OK) return r;
     std::swap(prev, cur);
     sig = sn;
@@ -434,6 +471,9 @@ cs_status cheb_ritz_dispatch(cs_ctx* c, int n_s, double* X, long long ld, const 
     case CS_FP64:
       return cheb_ritz_core<double>(c, n_s, X, ld, HX, ldh, theta, degree, a, b, a0, work, st);
     case CS_DF64:
+      if (c->n_p == 0 && use_sliced(c, n_s, true))
+        return cheb_ritz_core<double>(c, n_s, X, ld, HX, ldh, theta, degree, a, b, a0, work, st,
+                                      false, true);
       return cheb_ritz_core<df64>(c, n_s, X, ld, HX, ldh, theta, degree, a, b, a0, work, st);
     case CS_FP32:
     case CS_MIXED_BF16:
@@ -504,13 +544,19 @@ cs_status rr_core(cs_ctx* c, int n_s, double* X, long long ld, double* theta, do
   double* Q = Hs + (size_t)n_s * n_s;
   double* jw = Q + (size_t)n_s * n_s;
   cs_status r;
+  // Above kOneCtaEig states the eigensolver works in FP64 throughout and the signs of its vectors
+  // follow the last bits of the projected matrix, so there the H X keeps the FMA kernels'
+  // rounding: X and HX_out would come back with other signs for the same block (880 states:
+  // 256 ms with the slice products, 494 without).
+  const bool fma = n_s > kOneCtaEig;
   if (c->rr_prec == CS_FP64) {
-    r = hx_core<double>(c, n_s, X, ld, HX, H.d, EP_APPLY, 0, 0, 0, nullptr, work, st);
+    r = hx_core<double>(c, n_s, X, ld, HX, H.d, EP_APPLY, 0, 0, 0, nullptr, work, st, false,
+                        nullptr, nullptr, nullptr, false, fma);
   } else if (c->rr_prec == CS_DF64) {
     // H X in double-float: block split into tmp, product into HX, widened in place
     df64* Xd = reinterpret_cast<df64*>(work + lay.tmp);
     df64* Yd = reinterpret_cast<df64*>(work + lay.HX);
-    r = hx_df64_from_fp64(c, n_s, X, ld, HX, H.d, Xd, Yd, work, st);
+    r = hx_df64_from_fp64(c, n_s, X, ld, HX, H.d, Xd, Yd, work, st, fma);
   } else {
     // H X in the reduced precision (FP32 block in X32, result in tmp), then back to FP64;
     // the projection, eigensolve, rotations and residual norms below stay FP64
@@ -546,7 +592,8 @@ cs_status rr_core(cs_ctx* c, int n_s, double* X, long long ld, double* theta, do
 }
 
 cs_status hx_df64_from_fp64(cs_ctx* c, int n_s, const double* X, long long ld, double* HX,
-                            long long ldh, df64* Xd, df64* Yd, char* work, cudaStream_t st) {
+                            long long ldh, df64* Xd, df64* Yd, char* work, cudaStream_t st,
+                            bool fma) {
   const HostTables& H = c->host;
   const Layout lay = layout(c, n_s, CS_FP64);
   const df64* kb = nullptr;
@@ -565,9 +612,13 @@ cs_status hx_df64_from_fp64(cs_ctx* c, int n_s, const double* X, long long ld, d
     CS_LAUNCH_CLS(c, prof_cls<df64>(4), 4,
                   launch_oz_rotate(c->d64.pcoef, H.d, Wkb, c->n_p, H.d, c->n_p, n_s, kbZ, H.d, oz,
                                    c->dev_err, st));
-    CS_LAUNCH(c, 1, launch_to_df64(kbZ, H.d, reinterpret_cast<df64*>(kbZ), H.d, H.d, n_s, st));
+    if (fma || !use_sliced(c, n_s, true))
+      CS_LAUNCH(c, 1, launch_to_df64(kbZ, H.d, reinterpret_cast<df64*>(kbZ), H.d, H.d, n_s, st));
     kb = reinterpret_cast<const df64*>(kbZ);
   }
+  if (!fma && use_sliced(c, n_s, true))  // the slice products take and give FP64 blocks
+    return hx_core<double>(c, n_s, X, ld, HX, ldh, EP_APPLY, 0, 0, 0, nullptr, work, st, false,
+                           nullptr, nullptr, reinterpret_cast<const double*>(kb), true);
   CS_LAUNCH(c, 1, launch_to_df64(X, ld, Xd, H.d, H.d, n_s, st));
   cs_status r = hx_core<df64>(c, n_s, Xd, H.d, Yd, H.d, EP_APPLY, 0, 0, 0, nullptr, work, st,
                               false, nullptr, nullptr, kb);
@@ -606,6 +657,8 @@ cs_status chfsi_step_core(cs_ctx* c, int n_s, double* X, long long ld, int degre
     s = cheb_ritz_dispatch(c, n_s, X, ld, ritz_HX, ldh, theta, degree, a, b, a0, prec, wk, st);
   } else if (prec == CS_FP64) {
     s = cheb_core<double>(c, n_s, X, ld, degree, a, b, a0, wk, st);
+  } else if (prec == CS_DF64 && c->n_p == 0 && use_sliced(c, n_s, true)) {
+    s = cheb_core<double>(c, n_s, X, ld, degree, a, b, a0, wk, st, false, true);
   } else if (prec == CS_DF64) {
     df64* Xd = reinterpret_cast<df64*>(wk + lay.tmp);
     CS_LAUNCH(c, 1, launch_to_df64(X, ld, Xd, H.d, H.d, n_s, st));
@@ -709,6 +762,12 @@ cs_status cs_basis_init(double R, int lmax, int nmax, const cs_quadrature* q, in
                 cudaSuccess)
           st = CS_ERR_ALLOC;
       }
+      if (st == CS_OK && sliced_hx_eligible(c->host.L, c->host.N, c->host.n_r, c->host.n_theta,
+                                            c->host.n_phi)) {
+        if (build_sliced_tables(c->host, c->d64.rad, c->d64.theta, c->sliced) != cudaSuccess)
+          st = CS_ERR_ALLOC;
+        c->sliced_ok = st == CS_OK;
+      }
       if (st == CS_OK && (cudaMalloc((void**)&c->dev_err, sizeof(int)) != cudaSuccess ||
                           cudaMemset(c->dev_err, 0, sizeof(int)) != cudaSuccess))
         st = CS_ERR_ALLOC;
@@ -773,6 +832,7 @@ cs_status cs_basis_free(cs_ctx* c) {
     if (c->tc_anal) cudaFree(c->tc_anal);
     if (c->tc_phi) cudaFree(c->tc_phi);
     if (c->wide_tab) cudaFree(c->wide_tab);
+    free_sliced_tables(c->sliced);
     if (c->kb_tabA) cudaFree(c->kb_tabA);
     if (c->kb_tabB) cudaFree(c->kb_tabB);
     if (c->dev_err) cudaFree(c->dev_err);
@@ -821,6 +881,8 @@ cs_status cs_set_potential(cs_ctx* c, const double* v_grid, cs_stream stream) {
   cudaStream_t st = (cudaStream_t)stream;
   CS_LAUNCH(c, 1, launch_weighted_potential(v_grid, c->d64.wkj, H.n_r * H.n_theta, H.n_phi,
                                             c->d64.wv, c->d32.wv, c->ddf.wv, st));
+  if (c->sliced_ok)
+    CS_LAUNCH(c, 1, launch_sliced_wv(c->sliced, c->d64.wv, H.n_r * H.n_theta, H.n_phi, st));
   c->has_potential = true;
   return CS_OK;
 }
@@ -991,6 +1053,8 @@ cs_status cs_cheb_filter(cs_ctx* c, int n_s, void* X, long long ld, int degree, 
   if (prec == CS_FP32 || prec == CS_MIXED_BF16)
     return cheb_core<float>(c, n_s, (float*)X, ld, degree, a, b, a0, (char*)work, st,
                             prec == CS_MIXED_BF16);
+  if (prec == CS_DF64 && c->n_p == 0 && use_sliced(c, n_s, true))
+    return cheb_core<double>(c, n_s, (double*)X, ld, degree, a, b, a0, (char*)work, st, false, true);
   if (prec == CS_DF64) {
     const HostTables& H = c->host;
     df64* Xd = reinterpret_cast<df64*>((char*)work + layout(c, n_s, CS_DF64).tmp);

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/cs.h"
+#include "sliced_hx.h"
 
 namespace cs {
 
@@ -75,6 +76,8 @@ struct cs_ctx {
   void* tc_synth = nullptr;  // split-BF16 radial tables (tensor-core path)
   void* tc_anal = nullptr;
   void* tc_phi = nullptr;    // split-BF16 phi operands of the tensor-core angular kernel
+  cs::SlicedTables sliced;   // integer slices of the tables (FP64 H.X on the tensor cores)
+  bool sliced_ok = false;
   void* wide_tab = nullptr;  // split-BF16 Legendre and folded-trig operands of the wide block
   int tc_rows_synth = 0, tc_kpad_synth = 0, tc_rows_anal = 0, tc_kpad_anal = 0;
   void* kb_tabA = nullptr;   // split-BF16 projector operands (kb_tc.cu), set with the projectors

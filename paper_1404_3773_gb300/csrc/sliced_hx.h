@@ -1,0 +1,42 @@
+// FP64 H.X from integer-slice products on the tensor cores (sliced_hx.cu; internal).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstddef>
+
+#include "hx_kernels.cuh"
+
+namespace cs {
+
+struct HostTables;
+
+// set-up tables of one basis, and W V of the current potential, as integer slices
+struct SlicedTables {
+  unsigned char* tab[6] = {};  // digit images of the six contractions' tables
+  int* exps = nullptr;         // table-row exponents: R1, then R2, L2 and the radial scaling
+  size_t off_f2 = 0, off_fl = 0, off_re = 0;
+  int F1 = 0;                  // exponent of the Legendre table of the synthesis
+  long long* wv = nullptr;     // [k][j][q] W V below the row's power of two
+  int* ewv = nullptr;          // [k][j]
+};
+
+// lmax <= 62, n_theta <= 128, n_phi <= 255 (64 table rows or K per class); N, n_r <= 448 (the
+// 64-bit sums of the radial products)
+bool sliced_hx_eligible(int L, int N, int n_r, int n_theta, int n_phi);
+// CS_ANGULAR_KERNEL (any value) keeps the FMA kernels
+bool sliced_hx_enabled();
+size_t sliced_hx_work_bytes(int L, int n_r, int n_theta, int n_phi, int S);
+// rad, theta: the FP64 device tables
+cudaError_t build_sliced_tables(const HostTables& H, const double* rad, const double* theta,
+                                SlicedTables& T);
+void free_sliced_tables(SlicedTables& T);
+cudaError_t launch_sliced_wv(const SlicedTables& T, const double* wv, int rows, int n_phi,
+                             cudaStream_t st);
+// stage 0: radial synthesis X -> G; 1: the angular block on G, in place; 2: radial analysis of G
+// with the epilogue. *launches receives the kernel count.
+cudaError_t launch_sliced_hx(const HostTables& H, const SlicedTables& T, int S, const double* X,
+                             long long ld, double* G, const Epilogue<double>& ep, void* work,
+                             int* err, cudaStream_t st, int stage, int* launches);
+
+}  // namespace cs

@@ -136,6 +136,13 @@ __device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, float* v) {
         "=r"(r[7])
       : "r"(taddr));
 }
+// 4 columns
+__device__ __forceinline__ void tmem_ld4_issue(uint32_t taddr, float* v) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
