@@ -40,8 +40,8 @@ cs_status cs_scf_workspace_bytes(const cs_ctx* ctx, size_t* bytes);
 /* rho[g] = 2 sum_s occ[s] psi_s(x_g)^2, with psi_s = B X[:, s] the inverse basis transform of
  * column s (eq. density_expression, spin-unpolarised; Sec. 2.2.5 transform method).
  * X: DEVICE FP64 d x n_s, leading dimension ld >= d. occ: DEVICE n_s doubles (0..1).
- * rho: DEVICE N_g doubles (written; no accumulation across calls). States are processed
- * CS_DENSITY_CHUNK at a time, and the sum over s runs in state order (deterministic). */
+ * rho: DEVICE N_g doubles (written; no accumulation across calls). States are processed in
+ * chunks, and the sum over s runs in state order (deterministic). */
 cs_status cs_density(cs_ctx* ctx, int n_s, const double* X, long long ld, const double* occ,
                      double* rho, void* work, cs_stream stream);
 

@@ -232,22 +232,6 @@ cs_status upload_tables(cs_ctx* c) {
   return CS_OK;
 }
 
-// Whether an FP64 (or, with df, a double-float) H.X of n_s states takes the slice products
-// (sliced_hx.cu), by the number of grid rows x states.
-// FP64: they are faster at every size measured (lmax 6 .. 60, 1 .. 130 states): 0.074 against
-// 0.092 ms at 3456 rows, where launches dominate, 0.084 against 0.134 at 5120, 1.50 against 7.13
-// at 460800 (lmax 30, 80 states). Below 4096 rows, with little to gain, the kernels that
-// cs_apply_H_noalloc runs stay.
-// Double-float: its kernels cost less per row at small lmax. rows L^2 = 14M is where the two
-// meet: 0.130 / 0.122 ms at 7.4M (lmax 16, 16 states), 0.177 / 0.181 at 15M (lmax 23, 8),
-// 0.168 / 0.193 at 15M (lmax 16, 32), 0.254 / 0.336 at 44M (lmax 30, 8).
-bool use_sliced(const cs_ctx* c, int n_s, bool df) {
-  if (!c->sliced_ok || !sliced_hx_enabled()) return false;
-  const HostTables& H = c->host;
-  const long long rows = (long long)H.n_r * H.n_theta * n_s;
-  return rows * H.L * H.L >= 14000000 || (!df && rows >= 4096);
-}
-
 // ------------------------------------------------------------------ H.X core
 // out = epilogue(1/2 Lambda X + Z (+ kb)); see Epilogue in hx_kernels.cuh
 template <typename T>
@@ -986,13 +970,19 @@ cs_status cs_forward_transform(cs_ctx* c, int n, const double* g, double* coef, 
   cudaStream_t st = (cudaStream_t)stream;
   const Layout lay = layout(c, n, CS_FP64);
   double* G = reinterpret_cast<double*>((char*)work + lay.G);
-  AngArgs<double> a{H.L, H.n_r, H.n_theta, H.n_phi, c->Q4, n, c->d64.theta, c->d64.trig,
-                    c->d64.wv, c->d64.wkj};
-  CS_LAUNCH(c, 1, launch_angular<double>(a, ANG_ANAL, G, nullptr, g, st));
   Epilogue<double> ep;
   ep.mode = EP_PLAIN;
   ep.out = coef;
   ep.ld_out = ld;
+  if (use_sliced(c, n, false)) {
+    int nl = 0;
+    CS_LAUNCH(c, nl, launch_sliced_forward(H, c->sliced, n, g, c->d64.wkj, G, ep,
+                                           (char*)work + lay.sl, c->dev_err, st, &nl));
+    return CS_OK;
+  }
+  AngArgs<double> a{H.L, H.n_r, H.n_theta, H.n_phi, c->Q4, n, c->d64.theta, c->d64.trig,
+                    c->d64.wv, c->d64.wkj};
+  CS_LAUNCH(c, 1, launch_angular<double>(a, ANG_ANAL, G, nullptr, g, st));
   CS_LAUNCH(c, 1, launch_radial_anal<double>(G, c->d64.rad, H.L, H.N, H.n_r, n, ep, st));
   return CS_OK;
 }
@@ -1007,6 +997,12 @@ cs_status cs_inverse_transform(cs_ctx* c, int n, const double* coef, long long l
   cudaStream_t st = (cudaStream_t)stream;
   const Layout lay = layout(c, n, CS_FP64);
   double* G = reinterpret_cast<double*>((char*)work + lay.G);
+  if (use_sliced(c, n, false)) {
+    int nl = 0;
+    CS_LAUNCH(c, nl, launch_sliced_grid(H, c->sliced, n, coef, ld, G, f, (char*)work + lay.sl,
+                                        c->dev_err, st, &nl));
+    return CS_OK;
+  }
   CS_LAUNCH(c, 1, launch_radial_synth<double>(coef, ld, G, c->d64.rad, H.L, H.N, H.n_r, n, st));
   AngArgs<double> a{H.L, H.n_r, H.n_theta, H.n_phi, c->Q4, n, c->d64.theta, c->d64.trig,
                     c->d64.wv, c->d64.wkj};

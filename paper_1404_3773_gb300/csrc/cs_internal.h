@@ -96,3 +96,23 @@ struct cs_ctx {
   std::vector<ProfRec> prof_recs;
   std::vector<cudaEvent_t> event_pool;
 };
+
+namespace cs {
+
+// Whether an FP64 (or, with df, a double-float) H.X of n_s states takes the slice products
+// (sliced_hx.cu), by the number of grid rows x states.
+// FP64: they are faster at every size measured (lmax 6 .. 60, 1 .. 130 states): 0.074 against
+// 0.092 ms at 3456 rows, where launches dominate, 0.084 against 0.134 at 5120, 1.50 against 7.13
+// at 460800 (lmax 30, 80 states). Below 4096 rows, with little to gain, the kernels that
+// cs_apply_H_noalloc runs stay.
+// Double-float: its kernels cost less per row at small lmax. rows L^2 = 14M is where the two
+// meet: 0.130 / 0.122 ms at 7.4M (lmax 16, 16 states), 0.177 / 0.181 at 15M (lmax 23, 8),
+// 0.168 / 0.193 at 15M (lmax 16, 32), 0.254 / 0.336 at 44M (lmax 30, 8).
+inline bool use_sliced(const cs_ctx* c, int n_s, bool df) {
+  if (!c->sliced_ok || !sliced_hx_enabled()) return false;
+  const HostTables& H = c->host;
+  const long long rows = (long long)H.n_r * H.n_theta * n_s;
+  return rows * H.L * H.L >= 14000000 || (!df && rows >= 4096);
+}
+
+}  // namespace cs

@@ -55,8 +55,13 @@ struct ScfLayout {
   size_t alm;      // L^2 doubles (harmonic-term amplitudes)
   size_t G1;       // N_r L^2 doubles (Hartree radial synthesis)
   size_t partial;  // kDotBlocks x CS_GRID_INTEGRALS_MAX doubles
+  size_t slG, slw; // radial synthesis and intermediates of kSlChunk states (slice products)
   size_t total;
 };
+
+// states per slice-product synthesis of the density; larger blocks fill the tiles' 128 rows and
+// the last wave better (80 states in 3 blocks of 27)
+constexpr int kSlChunk = 32;
 
 ScfLayout scf_layout(const cs_ctx* c) {
   ScfLayout o{};
@@ -76,6 +81,8 @@ ScfLayout scf_layout(const cs_ctx* c) {
   o.alm = take(L2 * 8);
   o.G1 = take((size_t)H.n_r * L2 * 8);
   o.partial = take((size_t)(kDotBlocks + 1) * CS_GRID_INTEGRALS_MAX * 8);  // partials, results
+  o.slG = take(c->sliced_ok ? (size_t)H.n_r * L2 * kSlChunk * 8 : 0);
+  o.slw = take(c->sliced_ok ? sliced_hx_work_bytes(H.L, H.n_r, H.n_theta, H.n_phi, kSlChunk) : 0);
   o.total = off;
   return o;
 }
@@ -385,6 +392,18 @@ cs_status cs_density(cs_ctx* c, int n_s, const double* X, long long ld, const do
   double* f = reinterpret_cast<double*>(w + lay.fgrid);
   const long long ng = n_grid(c);
   cudaStream_t st = (cudaStream_t)stream;
+  if (use_sliced(c, n_s, false)) {
+    const int nb = (n_s + kSlChunk - 1) / kSlChunk, per = (n_s + nb - 1) / nb;
+    for (int s0 = 0; s0 < n_s; s0 += per) {
+      int nl = 0;
+      SCF_CUDA(c, launch_sliced_density(c->host, c->sliced, std::min(per, n_s - s0),
+                                        X + (size_t)s0 * ld, ld, occ + s0, s0 > 0,
+                                        reinterpret_cast<double*>(w + lay.slG), rho, w + lay.slw,
+                                        c->dev_err, st, &nl));
+      c->launches += nl;
+    }
+    return CS_OK;
+  }
   for (int s0 = 0; s0 < n_s; s0 += CS_DENSITY_CHUNK) {
     const int nc = std::min(CS_DENSITY_CHUNK, n_s - s0);
     cs_status r = cs_inverse_transform(c, nc, X + (size_t)s0 * ld, ld, f, w + lay.trans, stream);
@@ -418,6 +437,13 @@ cs_status cs_hartree(cs_ctx* c, const double* rho, double* vh, void* work, cs_st
   k_hartree_radial<<<(H.n_r * L2 + 255) / 256, 256, 0, st>>>(coef, c->d64.rad, alm, rr, H.L,
                                                                H.N, H.n_r, G1);
   SCF_CUDA(c, cudaGetLastError());
+  if (use_sliced(c, 1, false)) {
+    int nl = 0;
+    SCF_CUDA(c, launch_sliced_grid(H, c->sliced, 1, nullptr, 0, G1, vh, w + lay.slw, c->dev_err, st,
+                                   &nl));
+    c->launches += 2 + nl;
+    return CS_OK;
+  }
   AngArgs<double> a{H.L, H.n_r, H.n_theta, H.n_phi, c->Q4, 1, c->d64.theta, c->d64.trig,
                     c->d64.wv, c->d64.wkj};
   SCF_CUDA(c, launch_angular<double>(a, ANG_SYNTH, G1, vh, nullptr, st));

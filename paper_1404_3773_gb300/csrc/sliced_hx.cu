@@ -732,6 +732,156 @@ __global__ void __launch_bounds__(256) k_sl_pointwise(long long* __restrict__ W,
   }
 }
 
+// The folded classes of grid functions g[s][k][j][q] times the row's quadrature weight, as the
+// pointwise pass leaves them: one warp per (grid row, state), lanes over the quarter angles.
+__global__ void __launch_bounds__(256) k_sl_fold(const double* __restrict__ g,
+                                                 const double* __restrict__ wkj, int rows, int SB,
+                                                 int s0, int k0, int Nt, int Np, int Q, int n_r,
+                                                 long long* __restrict__ W,
+                                                 int* __restrict__ shP, int* __restrict__ uP,
+                                                 int* __restrict__ U) {
+  const int lane = threadIdx.x & 31;
+  const long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= (long long)rows * SB) return;
+  const int row = (int)(i / SB), s = (int)(i - (long long)row * SB);
+  const long long gr = (long long)k0 * Nt + row;
+  const double* x = g + ((long long)(s0 + s) * n_r * Nt + gr) * Np;
+  const double wt = __ldg(wkj + gr);
+  const int h = Np / 2;
+  double v[2][4];
+  int mx = 0;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int q = lane + 32 * u;
+    const int at[4] = {q, q == 0 ? 0 : Np - q, h - q, h + q};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      v[u][c] = q < Q ? __ldg(x + at[c]) * wt : 0.0;
+      mx = max(mx, (int)((__double_as_longlong(v[u][c]) >> 52) & 0x7FF));
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  const int E = exp_above_bits(mx);
+  unsigned long long acc = 0;
+  long long* o = W + (size_t)row * 4 * Q * SB + s;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int q = lane + 32 * u;
+    if (q >= Q) continue;
+    long long f[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      f[c] = fix_f64((unsigned long long)__double_as_longlong(v[u][c]), E) * 2;
+    const int hf = (q == 0 || 2 * q == h) ? 1 : 0;
+    const long long P = (f[0] + f[1]) >> hf, M = (f[0] - f[1]) >> hf;
+    const long long P2 = (f[2] + f[3]) >> hf, N2 = (f[2] - f[3]) >> hf;
+    const long long r[4] = {P + P2, P - P2, M - N2, M + N2};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      o[(size_t)(c * Q + q) * SB] = r[c];
+      acc |= (unsigned long long)(r[c] ^ (r[c] >> 63));
+    }
+  }
+  const int bits = __reduce_max_sync(0xffffffffu, bit_len(acc));
+  if (lane == 0) {
+    const int sh = clamp_shift(bits);
+    const int u = E - kFix - 1 - sh + kFix - 56;
+    shP[i] = sh;
+    uP[i] = u;
+    if (bits || u > kNonFinite / 2) atomicMax(U + (row / Nt) * SB + s, u);
+  }
+}
+
+// Grid values f[s][k][j][q] from the class sums: one warp per (grid row, state), the CTA's warps
+// on consecutive states so that they share the sectors of W.
+__global__ void __launch_bounds__(256) k_sl_grid(const long long* __restrict__ W,
+                                                 const int* __restrict__ eW, int rows, int SB,
+                                                 int s0, int k0, int Nt, int Np, int Q, int n_r,
+                                                 double* __restrict__ f) {
+  const int lane = threadIdx.x & 31;
+  const long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= (long long)rows * SB) return;
+  const int row = (int)(i / SB), s = (int)(i - (long long)row * SB);
+  double* y = f + ((long long)(s0 + s) * n_r * Nt + (long long)k0 * Nt + row) * Np;
+  const long long* x = W + (size_t)row * 4 * Q * SB + s;
+  const size_t cs = (size_t)Q * SB;
+  const int h = Np / 2, u = eW[i];
+  for (int q = lane; q < Q; q += 32) {
+    const long long* p = x + (size_t)q * SB;
+    const long long c0 = __ldg(p), c1 = __ldg(p + cs), c2 = __ldg(p + 2 * cs),
+                    c3 = __ldg(p + 3 * cs);
+    const long long ep = c0 + c1, em = c0 - c1, op = c2 + c3, om = c2 - c3;
+    y[q] = to_f64(ep + op, u);
+    if (q > 0) y[Np - q] = to_f64(ep - op, u);
+    if (2 * q != h) {
+      y[h - q] = to_f64(em - om, u);
+      if (q > 0) y[h + q] = to_f64(em + om, u);
+    }
+  }
+}
+
+// rho (+)= 2 sum_s occ[s] f[s]^2 over the block's states, in state order. One CTA per grid row:
+// the four mirror angles of every quarter angle for 32 states at a time (lanes over the states),
+// through shared memory to one thread per angle. A state's power of two goes into its weight, so
+// that the squares need three FP64 operations per value; the FP64 pipe is what bounds this pass.
+__global__ void __launch_bounds__(256) k_sl_density(const long long* __restrict__ W,
+                                                    const int* __restrict__ eW, int SB, int Nt,
+                                                    int Np, int Q, int k0,
+                                                    const double* __restrict__ occ,
+                                                    double* __restrict__ rho, int accumulate) {
+  extern __shared__ double dsm[];  // [4 Q][33], then weights [32]
+  double* wt = dsm + 4 * Q * 33;
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int row = blockIdx.x, h = Np / 2;
+  const long long* x = W + (size_t)row * 4 * Q * SB;
+  const size_t cs = (size_t)Q * SB;
+  double acc = 0.0;  // the angle 4 q + c of this thread: at most 4 Q <= 256
+  for (int b = 0; b < SB; b += 32) {
+    const int s = b + lane;
+    const bool live = s < SB;
+    const int u = live ? eW[(size_t)row * SB + s] : 0;
+    const bool plain = u > -400 && u < 400;  // the square of the unit stays in range
+    __syncthreads();
+    if (wp == 0) {
+      const double o = live ? __ldg(occ + s) : 0.0;
+      wt[lane] = plain ? o * oz_pow2(2 * u) : o;
+    }
+    for (int q = wp; q < Q; q += 8) {
+      long long c0 = 0, c1 = 0, c2 = 0, c3 = 0;
+      if (live) {
+        const long long* p = x + (size_t)q * SB + s;
+        c0 = __ldg(p);
+        c1 = __ldg(p + cs);
+        c2 = __ldg(p + 2 * cs);
+        c3 = __ldg(p + 3 * cs);
+      }
+      const long long ep = c0 + c1, em = c0 - c1, op = c2 + c3, om = c2 - c3;
+      const long long f[4] = {ep + op, ep - op, em - om, em + om};
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        dsm[(4 * q + c) * 33 + lane] = plain ? (double)f[c] : to_f64(f[c], u);
+    }
+    __syncthreads();
+    if (tid < 4 * Q) {
+      const int n = min(32, SB - b);
+      for (int i = 0; i < n; ++i) {
+        const double v = dsm[tid * 33 + i];
+        acc = fma(wt[i] * v, v, acc);
+      }
+    }
+  }
+  if (tid < 4 * Q) {
+    const int q = tid >> 2, c = tid & 3;
+    const int p = c == 0 ? q : c == 1 ? Np - q : c == 2 ? h - q : h + q;
+    // mirror angles that coincide are written once
+    const bool own = c == 0 || (c == 1 && q > 0) || (c >= 2 && 2 * q != h && (c == 2 || q > 0));
+    if (own) {
+      double* o = rho + ((long long)k0 * Nt + row) * Np + p;
+      *o = (accumulate ? *o : 0.0) + 2.0 * acc;
+    }
+  }
+}
+
 // E_G[k][s]: 2^E above every |G[k][lm][s]|
 __global__ void __launch_bounds__(256) k_sl_gexp(const double* __restrict__ G, int L2, int S,
                                                  int* __restrict__ EG) {
@@ -892,7 +1042,7 @@ size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 
 size_t node_bytes(int L, int n_theta, int n_phi, int SB) {
   const size_t NP = (n_theta + 1) / 2, M2 = 2 * L - 1, Q = n_phi / 4 + 1;
-  return (2 * NP * M2 + (size_t)n_theta * 4 * Q) * SB * 8 + (size_t)n_theta * SB * 12;
+  return (2 * NP * M2 + (size_t)n_theta * 4 * Q) * SB * 8 + (size_t)n_theta * SB * 12 + SB * 4;
 }
 
 void chunking(int L, int n_r, int n_theta, int n_phi, int S, int& SB, int& kc) {
@@ -934,13 +1084,11 @@ bool sliced_hx_eligible(int L, int N, int n_r, int n_theta, int n_phi) {
 
 bool sliced_hx_enabled() { return getenv("CS_ANGULAR_KERNEL") == nullptr; }
 
+// An upper bound of what SlPlan takes that grows with S, so that a workspace sized for S states
+// serves every smaller block: at most n_r nodes, and at most kChunkBytes or one node.
 size_t sliced_hx_work_bytes(int L, int n_r, int n_theta, int n_phi, int S) {
-  int SB, kc;
-  chunking(L, n_r, n_theta, n_phi, S, SB, kc);
-  const size_t rows = (size_t)kc * n_theta * SB;
-  const size_t NP = (n_theta + 1) / 2, M2 = 2 * L - 1, Q = n_phi / 4 + 1;
-  return al((size_t)kc * 2 * NP * M2 * SB * 8) + al(rows * 4 * Q * 8) + 3 * al(rows * 4) +
-         al((size_t)kc * SB * 4) + al((size_t)n_r * S * 4);
+  const size_t node = node_bytes(L, n_theta, n_phi, std::min(S, kMaxSB));
+  return std::min((size_t)n_r * node, kChunkBytes + node) + (size_t)n_r * S * 4 + 7 * 256;
 }
 
 void free_sliced_tables(SlicedTables& T) {
@@ -1023,100 +1171,222 @@ cudaError_t launch_sliced_wv(const SlicedTables& T, const double* wv, int rows, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_sliced_hx(const HostTables& H, const SlicedTables& T, int S, const double* X,
-                             long long ld, double* G, const Epilogue<double>& ep, void* work,
-                             int* err, cudaStream_t st, int stage, int* launches) {
-  const int L = H.L, L2 = L * L, NP = (H.n_theta + 1) / 2, M2 = 2 * L - 1, Q = H.n_phi / 4 + 1;
-  const int halfm = (L + 1) / 2, nb2 = halfm <= 16 ? 16 : 32;
-  int SBm, kcm;
-  chunking(L, H.n_r, H.n_theta, H.n_phi, S, SBm, kcm);
-  char* p = static_cast<char*>(work);
-  auto take = [&](size_t b) {
-    char* at = p;
-    p += al(b);
-    return at;
-  };
-  const size_t mrows = (size_t)kcm * H.n_theta * SBm;
+namespace {
+
+// One block's launches: the arguments shared by all operations and the workspace's parts.
+struct SlPlan {
+  const HostTables& H;
+  const SlicedTables& T;
+  cudaStream_t st;
   SlArgs a{};
-  a.L = L;
-  a.N = H.N;
-  a.n_r = H.n_r;
-  a.Nt = H.n_theta;
-  a.NP = NP;
-  a.M2 = M2;
-  a.Q = Q;
-  a.S = S;
-  a.F1 = T.F1;
-  a.ks = (halfm + 15) / 16;
-  a.nb2 = nb2;
-  a.rexp = T.exps + T.off_re;
-  a.X = X;
-  a.ld = ld;
-  a.G = G;
-  a.FA = reinterpret_cast<long long*>(take((size_t)kcm * 2 * NP * M2 * SBm * 8));
-  a.W = reinterpret_cast<long long*>(take(mrows * 4 * Q * 8));
-  a.eW = reinterpret_cast<int*>(take(mrows * 4));
-  int* shP = reinterpret_cast<int*>(take(mrows * 4));
-  int* uP = reinterpret_cast<int*>(take(mrows * 4));
-  int* U = reinterpret_cast<int*>(take((size_t)kcm * SBm * 4));
-  int* EG = reinterpret_cast<int*>(take((size_t)H.n_r * S * 4));
-  a.shP = shP;
-  a.uP = uP;
-  a.U = U;
-  a.EG = EG;
-  a.err = err;
-  a.ep = ep;
-  auto G_ = [&](int op) { return geo(op, L, H.N, H.n_r, H.n_theta, H.n_phi); };
-  cudaError_t e;
+  int L2, Np, SBm, kcm, n = 0;  // n: kernels launched
+  int *shP, *uP, *U, *EG;
   long long rad_tiles = 0;
-  for (int l = 0; l < L; ++l) rad_tiles += ((long long)(2 * l + 1) * S + kRows - 1) / kRows;
-  *launches = 0;
-  if (stage == 0) {
+  Geo g[6];
+
+  SlPlan(const HostTables& H_, const SlicedTables& T_, int S, double* G, void* work, int* err,
+         cudaStream_t st_)
+      : H(H_), T(T_), st(st_), L2(H_.L * H_.L), Np(H_.n_phi) {
+    const int L = H.L, NP = (H.n_theta + 1) / 2, half = (L + 1) / 2;
+    for (int op = 0; op < 6; ++op) g[op] = geo(op, L, H.N, H.n_r, H.n_theta, H.n_phi);
+    chunking(L, H.n_r, H.n_theta, H.n_phi, S, SBm, kcm);
+    for (int l = 0; l < L; ++l) rad_tiles += ((long long)(2 * l + 1) * S + kRows - 1) / kRows;
+    char* p = static_cast<char*>(work);
+    auto take = [&](size_t b) {
+      char* at = p;
+      p += al(b);
+      return at;
+    };
+    const size_t mrows = (size_t)kcm * H.n_theta * SBm;
+    a.L = L;
+    a.N = H.N;
+    a.n_r = H.n_r;
+    a.Nt = H.n_theta;
+    a.NP = NP;
+    a.M2 = 2 * L - 1;
+    a.Q = Np / 4 + 1;
+    a.S = S;
+    a.F1 = T.F1;
+    a.ks = (half + 15) / 16;
+    a.nb2 = half <= 16 ? 16 : 32;
+    a.rexp = T.exps + T.off_re;
+    a.G = G;
+    a.FA = reinterpret_cast<long long*>(take((size_t)kcm * 2 * NP * a.M2 * SBm * 8));
+    a.W = reinterpret_cast<long long*>(take(mrows * 4 * a.Q * 8));
+    a.eW = reinterpret_cast<int*>(take(mrows * 4));
+    shP = reinterpret_cast<int*>(take(mrows * 4));
+    uP = reinterpret_cast<int*>(take(mrows * 4));
+    U = reinterpret_cast<int*>(take((size_t)kcm * SBm * 4));
+    EG = reinterpret_cast<int*>(take((size_t)H.n_r * S * 4));
+    a.shP = shP;
+    a.uP = uP;
+    a.U = U;
+    a.EG = EG;
+    a.err = err;
+  }
+  int rows() const { return a.kc * a.Nt; }  // grid rows of the chunk
+  long long row_tiles() const { return ((long long)rows() * a.SB + kRows - 1) / kRows; }
+  cudaError_t radial_synth(const double* X, long long ld) {
+    a.X = X;
+    a.ld = ld;
     a.tab = T.tab[OP_R1];
     a.fexp = T.exps;
     a.ntiles = rad_tiles;
-    *launches = 1;
-    return launch_sl<OP_R1, 32, false>(a, G_(OP_R1), st);
+    ++n;
+    return launch_sl<OP_R1, 32, false>(a, g[OP_R1], st);
   }
-  if (stage == 2) {
+  cudaError_t radial_anal(const Epilogue<double>& ep) {
+    a.ep = ep;
     a.tab = T.tab[OP_R2];
     a.fexp = T.exps + T.off_f2;
     a.ntiles = rad_tiles;
-    *launches = 1;
-    return launch_sl<OP_R2, 32, false>(a, G_(OP_R2), st);
+    ++n;
+    return launch_sl<OP_R2, 32, false>(a, g[OP_R2], st);
   }
-  k_sl_gexp<<<dim3((S + 31) / 32, H.n_r), 256, 0, st>>>(G, L2, S, EG);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  ++*launches;
-  for (int s0 = 0; s0 < S; s0 += SBm)
-    for (int k0 = 0; k0 < H.n_r; k0 += kcm) {
-      a.s0 = s0;
-      a.SB = std::min(SBm, S - s0);
-      a.k0 = k0;
-      a.kc = std::min(kcm, H.n_r - k0);
-      const int nodes = a.kc * a.SB, rows = a.kc * a.Nt * a.SB;
-      const long long leg = 2ll * ((nodes + kRows - 1) / kRows) +
-                            2ll * (L - 1) * ((2 * nodes + kRows - 1) / kRows);
-      const long long row_tiles = ((long long)rows + kRows - 1) / kRows;
-      if ((e = cudaMemsetAsync(U, 0x80, (size_t)nodes * sizeof(int), st)) != cudaSuccess) return e;
-      a.tab = T.tab[OP_L1];
-      a.ntiles = leg;
-      if ((e = launch_sl<OP_L1, 16, true>(a, G_(OP_L1), st)) != cudaSuccess) return e;
-      a.tab = T.tab[OP_P1];
-      a.ntiles = row_tiles;
-      if ((e = launch_sl<OP_P1, 16, true>(a, G_(OP_P1), st)) != cudaSuccess) return e;
-      k_sl_pointwise<<<(unsigned)((rows + 31) / 32), 256, 0, st>>>(
-          a.W, a.eW, T.wv, T.ewv, a.kc * a.Nt, a.SB, a.Nt, H.n_phi, Q, k0, shP, uP, U);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      a.tab = T.tab[OP_P2];
-      a.ntiles = 4 * row_tiles;
-      if ((e = launch_sl2<OP_P2>(a, G_(OP_P2), st)) != cudaSuccess) return e;
-      a.tab = T.tab[OP_L2];
-      a.fexp = T.exps + T.off_fl;
-      a.ntiles = leg;
-      if ((e = launch_sl2<OP_L2>(a, G_(OP_L2), st)) != cudaSuccess) return e;
-      *launches += 5;
-    }
+  cudaError_t scales() {
+    k_sl_gexp<<<dim3((a.S + 31) / 32, H.n_r), 256, 0, st>>>(a.G, L2, a.S, EG);
+    ++n;
+    return cudaGetLastError();
+  }
+  void legendre_tiles() {
+    const int nodes = a.kc * a.SB;
+    a.ntiles = 2ll * ((nodes + kRows - 1) / kRows) +
+               2ll * (a.L - 1) * ((2 * nodes + kRows - 1) / kRows);
+  }
+  // L1 and P1 of the chunk: the class sums of its grid rows in W
+  cudaError_t synth() {
+    legendre_tiles();
+    a.tab = T.tab[OP_L1];
+    n += 2;
+    cudaError_t e = launch_sl<OP_L1, 16, true>(a, g[OP_L1], st);
+    if (e != cudaSuccess) return e;
+    a.tab = T.tab[OP_P1];
+    a.ntiles = row_tiles();
+    return launch_sl<OP_P1, 16, true>(a, g[OP_P1], st);
+  }
+  // P2 and L2: from the folded W, its shifts and units to G'
+  cudaError_t anal() {
+    a.tab = T.tab[OP_P2];
+    a.ntiles = 4 * row_tiles();
+    n += 2;
+    cudaError_t e = launch_sl2<OP_P2>(a, g[OP_P2], st);
+    if (e != cudaSuccess) return e;
+    legendre_tiles();
+    a.tab = T.tab[OP_L2];
+    a.fexp = T.exps + T.off_fl;
+    return launch_sl2<OP_L2>(a, g[OP_L2], st);
+  }
+  cudaError_t clear_units() {
+    return cudaMemsetAsync(U, 0x80, (size_t)a.kc * a.SB * sizeof(int), st);
+  }
+  // body() for every block of states and chunk of radial nodes
+  template <class F>
+  cudaError_t chunks(F body) {
+    for (a.s0 = 0; a.s0 < a.S; a.s0 += SBm)
+      for (a.k0 = 0; a.k0 < H.n_r; a.k0 += kcm) {
+        a.SB = std::min(SBm, a.S - a.s0);
+        a.kc = std::min(kcm, H.n_r - a.k0);
+        const cudaError_t e = body();
+        if (e != cudaSuccess) return e;
+      }
+    return cudaSuccess;
+  }
+};
+
+unsigned warp_grid(long long items) { return (unsigned)((items + 7) / 8); }
+
+#define SL_TRY(expr)                          \
+  do {                                        \
+    const cudaError_t e_ = (expr);            \
+    if (e_ != cudaSuccess) return e_;         \
+  } while (0)
+
+}  // namespace
+
+cudaError_t launch_sliced_hx(const HostTables& H, const SlicedTables& T, int S, const double* X,
+                             long long ld, double* G, const Epilogue<double>& ep, void* work,
+                             int* err, cudaStream_t st, int stage, int* launches) {
+  SlPlan p(H, T, S, G, work, err, st);
+  SlArgs& a = p.a;
+  cudaError_t e;
+  if (stage == 0) {
+    e = p.radial_synth(X, ld);
+  } else if (stage == 2) {
+    e = p.radial_anal(ep);
+  } else {
+    SL_TRY(p.scales());
+    e = p.chunks([&]() -> cudaError_t {
+      SL_TRY(p.clear_units());
+      SL_TRY(p.synth());
+      const int rows = p.rows();
+      k_sl_pointwise<<<(unsigned)(((long long)rows * a.SB + 31) / 32), 256, 0, st>>>(
+          a.W, a.eW, T.wv, T.ewv, rows, a.SB, a.Nt, p.Np, a.Q, a.k0, p.shP, p.uP, p.U);
+      ++p.n;
+      SL_TRY(cudaGetLastError());
+      return p.anal();
+    });
+  }
+  *launches = p.n;
+  return e;
+}
+
+cudaError_t launch_sliced_grid(const HostTables& H, const SlicedTables& T, int S, const double* X,
+                               long long ld, double* G, double* f, void* work, int* err,
+                               cudaStream_t st, int* launches) {
+  SlPlan p(H, T, S, G, work, err, st);
+  SlArgs& a = p.a;
+  if (X) SL_TRY(p.radial_synth(X, ld));
+  SL_TRY(p.scales());
+  SL_TRY(p.chunks([&]() -> cudaError_t {
+    SL_TRY(p.synth());
+    const int rows = p.rows();
+    k_sl_grid<<<warp_grid((long long)rows * a.SB), 256, 0, st>>>(a.W, a.eW, rows, a.SB, a.s0, a.k0,
+                                                                 a.Nt, p.Np, a.Q, H.n_r, f);
+    ++p.n;
+    return cudaGetLastError();
+  }));
+  *launches = p.n;
+  return cudaSuccess;
+}
+
+cudaError_t launch_sliced_density(const HostTables& H, const SlicedTables& T, int S,
+                                  const double* X, long long ld, const double* occ, bool add,
+                                  double* G, double* rho, void* work, int* err, cudaStream_t st,
+                                  int* launches) {
+  SlPlan p(H, T, S, G, work, err, st);
+  SlArgs& a = p.a;
+  SL_TRY(p.radial_synth(X, ld));
+  SL_TRY(p.scales());
+  const int smem = (4 * a.Q * 33 + 32) * (int)sizeof(double);
+  SL_TRY(cudaFuncSetAttribute(k_sl_density, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  SL_TRY(p.chunks([&]() -> cudaError_t {
+    SL_TRY(p.synth());
+    k_sl_density<<<(unsigned)p.rows(), 256, smem, st>>>(a.W, a.eW, a.SB, a.Nt, p.Np, a.Q, a.k0,
+                                                       occ + a.s0, rho, add || a.s0 > 0 ? 1 : 0);
+    ++p.n;
+    return cudaGetLastError();
+  }));
+  *launches = p.n;
+  return cudaSuccess;
+}
+
+cudaError_t launch_sliced_forward(const HostTables& H, const SlicedTables& T, int S,
+                                  const double* g, const double* wkj, double* G,
+                                  const Epilogue<double>& ep, void* work, int* err,
+                                  cudaStream_t st, int* launches) {
+  SlPlan p(H, T, S, G, work, err, st);
+  SlArgs& a = p.a;
+  SL_TRY(p.chunks([&]() -> cudaError_t {
+    SL_TRY(p.clear_units());
+    const int rows = p.rows();
+    k_sl_fold<<<warp_grid((long long)rows * a.SB), 256, 0, st>>>(
+        g, wkj, rows, a.SB, a.s0, a.k0, a.Nt, p.Np, a.Q, H.n_r, a.W, p.shP, p.uP, p.U);
+    ++p.n;
+    SL_TRY(cudaGetLastError());
+    return p.anal();
+  }));
+  SL_TRY(p.radial_anal(ep));
+  *launches = p.n;
   return cudaSuccess;
 }
 

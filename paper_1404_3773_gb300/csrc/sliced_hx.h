@@ -39,4 +39,19 @@ cudaError_t launch_sliced_hx(const HostTables& H, const SlicedTables& T, int S, 
                              long long ld, double* G, const Epilogue<double>& ep, void* work,
                              int* err, cudaStream_t st, int stage, int* launches);
 
+// Grid values f[s][k][j][q] of S columns of X, or, with X null, of the radial synthesis in G.
+cudaError_t launch_sliced_grid(const HostTables& H, const SlicedTables& T, int S, const double* X,
+                               long long ld, double* G, double* f, void* work, int* err,
+                               cudaStream_t st, int* launches);
+// rho (+)= 2 sum_s occ[s] f[s]^2, in state order
+cudaError_t launch_sliced_density(const HostTables& H, const SlicedTables& T, int S,
+                                  const double* X, long long ld, const double* occ, bool add,
+                                  double* G, double* rho, void* work, int* err, cudaStream_t st,
+                                  int* launches);
+// Analysis of S grid functions g[s][k][j][q] times the row weights wkj, with the epilogue.
+cudaError_t launch_sliced_forward(const HostTables& H, const SlicedTables& T, int S,
+                                  const double* g, const double* wkj, double* G,
+                                  const Epilogue<double>& ep, void* work, int* err,
+                                  cudaStream_t st, int* launches);
+
 }  // namespace cs

@@ -133,3 +133,40 @@ def test_sliced_hx_scales(scale, monkeypatch):
     cs.cs_apply_H(ctx, to_dev(X * scale), out, cs.CS_FP64)
     fro, _ = rel_errors(to_host(out, ctx.d) / scale, to_host(ref, ctx.d))
     assert np.isfinite(fro) and fro <= CLOSE, fro
+
+
+@pytest.mark.parametrize("case", list(EDGES))
+def test_sliced_transforms_and_density_match_fma_kernels(case, monkeypatch):
+    """The transforms, the density (in blocks of states) and the Hartree potential (one state)
+    through the same passes; rows of zeros in the grid functions."""
+    torch, cs = need_gpu()
+    monkeypatch.delenv("CS_ANGULAR_KERNEL", raising=False)
+    w = _work(case)
+    ctx = make_ctx(w)
+    X = to_dev(w.x_block(), ld=ctx.d + 1)
+    shape = (w.n_s, ctx.n_r, ctx.n_theta, ctx.n_phi)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    g = torch.randn(shape, dtype=torch.float64, device="cuda", generator=gen)
+    g[:, 1, 2] = 0.0
+    g[0] = 0.0
+    occ = torch.rand(w.n_s, dtype=torch.float64, device="cuda", generator=gen)
+
+    def run():
+        coef = torch.zeros_like(X)
+        cs.cs_forward_transform(ctx, g, coef)
+        f = torch.zeros(shape, dtype=torch.float64, device="cuda")
+        cs.cs_inverse_transform(ctx, X, f)
+        rho, vh = torch.zeros_like(f[0]), torch.zeros_like(f[0])
+        cs.cs_density(ctx, X, occ, rho)
+        cs.cs_hartree(ctx, rho, vh)
+        return coef, f, rho, vh
+
+    got = run()
+    monkeypatch.setenv("CS_ANGULAR_KERNEL", "fma")
+    ref = run()
+    assert torch.all(got[0][0] == 0)
+    for name, a, b in zip(("forward", "inverse", "density", "hartree"), got, ref):
+        rel = float((a - b).norm() / b.norm())
+        print(f"sliced {name} {case}: {rel:.2e}")
+        assert rel <= CLOSE, (name, rel)
+    assert cs.cs_device_error(ctx) == 0
