@@ -719,6 +719,37 @@ __global__ void __launch_bounds__(1024) k_sym_eig(const double* __restrict__ Ain
     const T glo = bnd[0], ghi = bnd[1];
     const T tnorm = fmax(fabs(glo), fabs(ghi)) + T(1e-30);
     const T piv = eps * tnorm;  // pivot guard of the Sturm and LDL^T recurrences
+    // start vector differing per eigenvalue (and per attempt), so that a cluster's members start
+    // apart
+    auto start = [&](T* y, int i, int seed) {
+      for (int j = 0; j < n; ++j) {
+        const unsigned hsh = (unsigned)(j + 1) * 2654435761u ^
+                             (unsigned)(i + 1 + seed * 7919) * 40503u;
+        y[j] = T(0.5) + (T)((hsh >> 8) & 0xffffu) * T(1.0 / 65536.0);
+      }
+    };
+    // y <- (T - x)^-1 y, normalised, by the LDL^T factors of T - x (L: n values of scratch)
+    auto solve = [&](T* y, T* L, T x) {
+      T Dp = d[0] - x;
+      if (fabs(Dp) < piv) Dp = piv;
+      T zp = y[0];
+      y[0] = zp / Dp;
+      for (int j = 1; j < n; ++j) {
+        const T l = e[j - 1] / Dp;
+        L[j] = l;
+        const T z = y[j] - l * zp;
+        T Dj = d[j] - x - l * e[j - 1];
+        if (fabs(Dj) < piv) Dj = piv;
+        y[j] = z / Dj;
+        zp = z;
+        Dp = Dj;
+      }
+      for (int j = n - 2; j >= 0; --j) y[j] -= L[j + 1] * y[j + 1];
+      T ss = T(0);
+      for (int j = 0; j < n; ++j) ss += y[j] * y[j];
+      const T sc = rsqrt(ss);
+      for (int j = 0; j < n; ++j) y[j] *= sc;
+    };
     for (int i = tid; i < n; i += nt) {
       T a = glo - piv, b = ghi + piv;  // count(a) <= i < count(b)
       for (int it = 0; it < 64; ++it) {
@@ -740,32 +771,8 @@ __global__ void __launch_bounds__(1024) k_sym_eig(const double* __restrict__ Ain
       lam[i] = x;
       T* y = Y + (size_t)i * n;
       T* L = Ls + (size_t)i * n;
-      // start vector differing per eigenvalue, so that a cluster's members start apart
-      for (int j = 0; j < n; ++j) {
-        const unsigned hsh = (unsigned)(j + 1) * 2654435761u ^ (unsigned)(i + 1) * 40503u;
-        y[j] = T(0.5) + (T)((hsh >> 8) & 0xffffu) * T(1.0 / 65536.0);
-      }
-      for (int rep = 0; rep < 3; ++rep) {
-        T Dp = d[0] - x;
-        if (fabs(Dp) < piv) Dp = piv;
-        T zp = y[0];
-        y[0] = zp / Dp;
-        for (int j = 1; j < n; ++j) {
-          const T l = e[j - 1] / Dp;
-          L[j] = l;
-          const T z = y[j] - l * zp;
-          T Dj = d[j] - x - l * e[j - 1];
-          if (fabs(Dj) < piv) Dj = piv;
-          y[j] = z / Dj;
-          zp = z;
-          Dp = Dj;
-        }
-        for (int j = n - 2; j >= 0; --j) y[j] -= L[j + 1] * y[j + 1];
-        T ss = T(0);
-        for (int j = 0; j < n; ++j) ss += y[j] * y[j];
-        const T sc = rsqrt(ss);
-        for (int j = 0; j < n; ++j) y[j] *= sc;
-      }
+      start(y, i, 0);
+      for (int rep = 0; rep < 3; ++rep) solve(y, L, x);
     }
     __syncthreads();
     // clusters of eigenvalues closer than 1e-5 |T|: modified Gram-Schmidt, twice
@@ -786,14 +793,28 @@ __global__ void __launch_bounds__(1024) k_sym_eig(const double* __restrict__ Ain
         for (int i = tid; i < n; i += nt) {
           if (i - cst[i] != pos) continue;
           T* y = Y + (size_t)i * n;
-          for (int jv = cst[i]; jv < i; ++jv) {
-            const T* u = Y + (size_t)jv * n;
-            T dot = T(0);
-            for (int j = 0; j < n; ++j) dot += u[j] * y[j];
-            for (int j = 0; j < n; ++j) y[j] -= dot * u[j];
+          // y minus its components along the cluster's earlier members; what is left of |y|^2
+          auto project = [&]() -> T {
+            for (int jv = cst[i]; jv < i; ++jv) {
+              const T* u = Y + (size_t)jv * n;
+              T dot = T(0);
+              for (int j = 0; j < n; ++j) dot += u[j] * y[j];
+              for (int j = 0; j < n; ++j) y[j] -= dot * u[j];
+            }
+            T ss = T(0);
+            for (int j = 0; j < n; ++j) ss += y[j] * y[j];
+            return ss;
+          };
+          T ss = project();
+          // Equal eigenvalues to the last bit can give equal vectors: what is left is rounding
+          // noise, or nothing. Such a member starts again from another vector, kept away from
+          // the earlier members before and after its inverse iteration.
+          for (int at = 1; at <= 4 && !(ss > T(1e-8)); ++at) {
+            start(y, i, at);
+            project();
+            if (at < 4) solve(y, Ls + (size_t)i * n, lam[i]);
+            ss = project();
           }
-          T ss = T(0);
-          for (int j = 0; j < n; ++j) ss += y[j] * y[j];
           const T sc = rsqrt(ss);
           for (int j = 0; j < n; ++j) y[j] *= sc;
         }
