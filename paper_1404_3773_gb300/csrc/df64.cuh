@@ -146,6 +146,42 @@ struct df64acc {
 };
 __device__ __forceinline__ df64& operator-=(df64& a, df64 b) { return a = a - b; }
 
+// Two df64acc side by side on packed FP32 instructions (sm_100: one instruction, two lanes): the
+// same roundings per lane, half the instruction issue that bounds the double-float products.
+// Operands come as pairs of leading and trailing parts; nah = -ah, so that -p is a plain product.
+struct df64acc2 {
+  float2 hi = {0.f, 0.f}, lo = {0.f, 0.f};
+  __device__ __forceinline__ void add_prod(float2 ah, float2 nah, float2 al, float2 bh,
+                                           float2 bl) {
+    add(__fmul2_rn(nah, bh), ah, al, bh, bl);
+  }
+  // the same with -bh at hand
+  __device__ __forceinline__ void add_prod_nb(float2 ah, float2 al, float2 bh, float2 nbh,
+                                              float2 bl) {
+    add(__fmul2_rn(ah, nbh), ah, al, bh, bl);
+  }
+  // np = -p = -(ah bh) rounded
+  __device__ __forceinline__ void add(float2 np, float2 ah, float2 al, float2 bh, float2 bl) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    float2 e = __ffma2_rn(ah, bh, np);
+    e = __ffma2_rn(ah, bl, e);
+    e = __ffma2_rn(al, bh, e);
+    const float2 s = __ffma2_rn(np, m1, hi);   // hi + p
+    const float2 bb = __ffma2_rn(hi, m1, s);   // s - hi
+    const float2 t = __ffma2_rn(bb, m1, s);    // s - bb
+    const float2 u = __ffma2_rn(t, m1, hi);    // hi - (s - bb)
+    const float2 err = __ffma2_rn(__fadd2_rn(np, bb), m1, u);  // u + (p - bb)
+    hi = s;
+    lo = __fadd2_rn(lo, __fadd2_rn(err, e));
+  }
+  __device__ __forceinline__ df64 value(int lane) const {
+    df64acc a;
+    a.hi = lane ? hi.y : hi.x;
+    a.lo = lane ? lo.y : lo.x;
+    return a.value();
+  }
+};
+
 // Multiply-add accumulator over an arithmetic type: a fused multiply-add for float and double,
 // df64acc for df64 (one renormalisation when read).
 template <typename C>

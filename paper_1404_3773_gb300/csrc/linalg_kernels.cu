@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
+#include <type_traits>
 #include <utility>
 
 #include "df64.cuh"
@@ -52,8 +53,10 @@ __device__ __forceinline__ double out_val(double v) { return v; }
 __device__ __forceinline__ float out_val(float v) { return v; }
 __device__ __forceinline__ double out_val(df64 v) { return v.to_double(); }
 
-// F: storage type of A, B and the partials; C: arithmetic (F, or df64 for F = double)
-template <typename F, typename C, int U>
+// F: storage type of A, B and the partials; C: arithmetic (F, or df64 for F = double).
+// SYM (A and B are one block, one tile): only the 16 x 16 sub-blocks on and above the diagonal,
+// U (U + 1) / 2 of U^2; k_gram_reduce mirrors them.
+template <typename F, typename C, int U, bool SYM>
 __global__ void __launch_bounds__(256) k_gram_partial(const F* __restrict__ A, long long lda,
                                                        const F* __restrict__ B,
                                                        long long ldb, long long d, int na,
@@ -65,7 +68,7 @@ __global__ void __launch_bounds__(256) k_gram_partial(const F* __restrict__ A, l
   const long long r0 = (long long)chunk * rows;
   const long long r1 = min(d, r0 + rows);
   __shared__ C As[GK][T + 1];
-  __shared__ C Bs[GK][T + 1];
+  __shared__ C Bs[SYM ? 1 : GK][SYM ? 1 : T + 1];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   MacAcc<C> acc[U][U];
   for (long long rb = r0; rb < r1; rb += GK) {
@@ -74,7 +77,7 @@ __global__ void __launch_bounds__(256) k_gram_partial(const F* __restrict__ A, l
       long long r = rb + rr;
       int i = i0 + cc, j = j0 + cc;
       As[rr][cc] = (r < r1 && i < na) ? C(A[r + (long long)i * lda]) : C(0);
-      Bs[rr][cc] = (r < r1 && j < nb) ? C(B[r + (long long)j * ldb]) : C(0);
+      if (!SYM) Bs[rr][cc] = (r < r1 && j < nb) ? C(B[r + (long long)j * ldb]) : C(0);
     }
     __syncthreads();
 #pragma unroll
@@ -83,11 +86,11 @@ __global__ void __launch_bounds__(256) k_gram_partial(const F* __restrict__ A, l
 #pragma unroll
       for (int u = 0; u < U; ++u) a[u] = As[rr][tx + 16 * u];
 #pragma unroll
-      for (int v = 0; v < U; ++v) b[v] = Bs[rr][ty + 16 * v];
+      for (int v = 0; v < U; ++v) b[v] = SYM ? As[rr][ty + 16 * v] : Bs[rr][ty + 16 * v];
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int v = 0; v < U; ++v) acc[u][v].add_prod(a[u], b[v]);
+        for (int v = SYM ? u : 0; v < U; ++v) acc[u][v].add_prod(a[u], b[v]);
     }
     __syncthreads();
   }
@@ -95,23 +98,90 @@ __global__ void __launch_bounds__(256) k_gram_partial(const F* __restrict__ A, l
 #pragma unroll
   for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int v = 0; v < U; ++v) {
+    for (int v = SYM ? u : 0; v < U; ++v) {
       int i = i0 + tx + 16 * u, j = j0 + ty + 16 * v;
       if (i < na && j < nb) P[i + (size_t)j * na] = out_val(acc[u][v].value());
     }
 }
 
-// 32 elements x 8 chunk slices per 256-thread block; slices summed in a fixed order
+// The double-float Gram tile on packed FP32 instructions: a thread keeps two sums per entry, over
+// the even and the odd rows, so that a pair of neighbouring rows is one operand pair as it lies in
+// shared memory ([column][row], leading and trailing parts apart). d = 46128, 80 columns: X^T X
+// 0.204 ms in the scalar form (0.112 with the sub-blocks below the diagonal left out).
+template <int U, bool SYM>
+__global__ void __launch_bounds__(256) k_gram_partial_df(const double* __restrict__ A,
+                                                         long long lda,
+                                                         const double* __restrict__ B,
+                                                         long long ldb, long long d, int na,
+                                                         int nb, long long rows,
+                                                         double* __restrict__ partial) {
+  constexpr int T = 16 * U, P = GK + 2;
+  const int i0 = blockIdx.x * T, j0 = blockIdx.y * T;
+  const long long r0 = (long long)blockIdx.z * rows;
+  const long long r1 = min(d, r0 + rows);
+  __shared__ __align__(8) float Ah[T][P], Al[T][P];
+  __shared__ __align__(8) float Bh[SYM ? 1 : T][P], Bl[SYM ? 1 : T][P];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  df64acc2 acc[U][U];
+  for (long long rb = r0; rb < r1; rb += GK) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {  // GK T values, 256 threads
+      const int rr = tx, cc = ty + 16 * u;
+      const long long r = rb + rr;
+      const df64 x((r < r1 && i0 + cc < na) ? A[r + (long long)(i0 + cc) * lda] : 0.0);
+      Ah[cc][rr] = x.hi;
+      Al[cc][rr] = x.lo;
+      if (!SYM) {
+        const df64 y((r < r1 && j0 + cc < nb) ? B[r + (long long)(j0 + cc) * ldb] : 0.0);
+        Bh[cc][rr] = y.hi;
+        Bl[cc][rr] = y.lo;
+      }
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int rr = 0; rr < GK; rr += 2) {
+      float2 bh[U], bl[U];
+#pragma unroll
+      for (int v = 0; v < U; ++v) {
+        bh[v] = *reinterpret_cast<const float2*>(&(SYM ? Ah : Bh)[ty + 16 * v][rr]);
+        bl[v] = *reinterpret_cast<const float2*>(&(SYM ? Al : Bl)[ty + 16 * v][rr]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float2 ah = *reinterpret_cast<const float2*>(&Ah[tx + 16 * u][rr]);
+        const float2 al = *reinterpret_cast<const float2*>(&Al[tx + 16 * u][rr]);
+        const float2 nah = make_float2(-ah.x, -ah.y);
+#pragma unroll
+        for (int v = SYM ? u : 0; v < U; ++v) acc[u][v].add_prod(ah, nah, al, bh[v], bl[v]);
+      }
+    }
+    __syncthreads();
+  }
+  double* Pt = partial + (size_t)blockIdx.z * na * nb;
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = SYM ? u : 0; v < U; ++v) {
+      const int i = i0 + tx + 16 * u, j = j0 + ty + 16 * v;
+      if (i < na && j < nb)
+        Pt[i + (size_t)j * na] = (acc[u][v].value(0) + acc[u][v].value(1)).to_double();
+    }
+}
+
+// 32 elements x 8 chunk slices per 256-thread block; slices summed in a fixed order; sym: the
+// entries below the diagonal from those above
 template <typename F>
 __global__ void k_gram_reduce(const F* __restrict__ partial, int chunks, int na, int nb,
-                              F* __restrict__ C, int ldc) {
+                              F* __restrict__ C, int ldc, int sym) {
   __shared__ F red[8][33];
   const int el = threadIdx.x & 31, sl = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + el;
   const int E = na * nb;
   F s = F(0);
+  const int ei = e % na, ej = e / na;
+  const int src = sym && ei > ej ? ej + ei * na : e;
   if (e < E)
-    for (int c = sl; c < chunks; c += 8) s += partial[(size_t)c * E + e];
+    for (int c = sl; c < chunks; c += 8) s += partial[(size_t)c * E + src];
   red[sl][el] = s;
   __syncthreads();
   if (sl == 0 && e < E) {
@@ -129,16 +199,37 @@ static cudaError_t gram_impl(const F* A, long long lda, const F* B, long long ld
   long long rows;
   gram_shape(d, na, nb, u, ta, tb, chunks, rows);
   dim3 grid(ta, tb, chunks);
+  // X^T X of one tile (up to 96 columns): 15 of 25 sub-blocks at 80 columns
+  const bool sym = A == B && lda == ldb && na == nb && ta == 1;
+#define CS_GRAM_CASE(UV)                                                                        \
+  case UV:                                                                                      \
+    if constexpr (std::is_same<C, df64>::value && UV < 6) {                                     \
+      if (sym)                                                                                  \
+        k_gram_partial_df<UV, true><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows,  \
+                                                              partial);                         \
+      else                                                                                      \
+        k_gram_partial_df<UV, false><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, \
+                                                               partial);                        \
+    } else if (sym)                                                                                    \
+      k_gram_partial<F, C, UV, true><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, \
+                                                               partial);                        \
+    else                                                                                        \
+      k_gram_partial<F, C, UV, false><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, \
+                                                                partial);                       \
+    break;
   switch (u) {
-    case 1: k_gram_partial<F, C, 1><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, partial); break;
-    case 2: k_gram_partial<F, C, 2><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, partial); break;
-    case 3: k_gram_partial<F, C, 3><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, partial); break;
-    case 4: k_gram_partial<F, C, 4><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, partial); break;
-    case 5: k_gram_partial<F, C, 5><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, partial); break;
-    default: k_gram_partial<F, C, 6><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, partial); break;
+    CS_GRAM_CASE(1)
+    CS_GRAM_CASE(2)
+    CS_GRAM_CASE(3)
+    CS_GRAM_CASE(4)
+    CS_GRAM_CASE(5)
+    default:
+      CS_GRAM_CASE(6)
   }
+#undef CS_GRAM_CASE
   int tot = na * nb;
-  k_gram_reduce<F><<<(tot + 31) / 32, 256, 0, stream>>>(partial, chunks, na, nb, Cout, ldc);
+  k_gram_reduce<F><<<(tot + 31) / 32, 256, 0, stream>>>(partial, chunks, na, nb, Cout, ldc,
+                                                        sym ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -156,7 +247,9 @@ cudaError_t launch_gram_df(const double* A, long long lda, const double* B, long
 
 // ------------------------------------------------------------------ C = alpha A Q + beta C
 // 64 rows x (16U) columns per CTA; U from n so that 80 states are one column tile.
-template <typename F, typename Cm, int U>
+// UPPER: Q is upper triangular with zeros stored below its diagonal, so a step of 16 rows k of Q
+// meets only the column groups of 16 that reach it (15 of 25 at 80 columns).
+template <typename F, typename Cm, int U, bool UPPER>
 __global__ void __launch_bounds__(256) k_gemm_nn(const F* __restrict__ A, long long lda,
                                                   const F* __restrict__ Q, int ldq,
                                                   long long d, int K, int n, F alpha,
@@ -168,7 +261,9 @@ __global__ void __launch_bounds__(256) k_gemm_nn(const F* __restrict__ A, long l
   __shared__ Cm Qs[GK][BN + 1];  // Qs[k][j]
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   MacAcc<Cm> acc[4][U];
-  for (int k0 = 0; k0 < K; k0 += GK) {
+  const int kend = UPPER ? min(K, j0 + BN) : K;
+  for (int k0 = 0; k0 < kend; k0 += GK) {
+    const int v0 = UPPER ? max(0, (k0 - j0) / 16) : 0;  // first column group that k0 reaches
     for (int idx = tid; idx < GK * BM; idx += 256) {
       int rr = idx % BM, kk = idx / BM;
       long long r = r0 + rr;
@@ -189,9 +284,11 @@ __global__ void __launch_bounds__(256) k_gemm_nn(const F* __restrict__ A, long l
 #pragma unroll
       for (int v = 0; v < U; ++v) b[v] = Qs[kk][ty + 16 * v];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int v = 0; v < U; ++v) {
+        if (UPPER && v < v0) continue;
 #pragma unroll
-        for (int v = 0; v < U; ++v) acc[u][v].add_prod(a[u], b[v]);
+        for (int u = 0; u < 4; ++u) acc[u][v].add_prod(a[u], b[v]);
+      }
     }
     __syncthreads();
   }
@@ -211,34 +308,127 @@ __global__ void __launch_bounds__(256) k_gemm_nn(const F* __restrict__ A, long l
   }
 }
 
+// The double-float rotation on packed FP32 instructions: a thread owns 4 consecutive rows (two
+// operand pairs as they lie in shared memory) x U columns; the factor's values are stored twice
+// over, so that one 16-byte load gives both broadcast pairs. UPPER as in k_gemm_nn.
+template <int U, int V0>
+__device__ __forceinline__ void nn_df_step(const float* Ah, const float* Al, const float4* Qs,
+                                           int tx, int ty, df64acc2 (&acc)[2][U]) {
+  constexpr int BM = 64, BN = 16 * U;
+#pragma unroll 4
+  for (int kk = 0; kk < GK; ++kk) {
+    const float4 h = *reinterpret_cast<const float4*>(Ah + kk * (BM + 4) + 4 * tx);
+    const float4 l = *reinterpret_cast<const float4*>(Al + kk * (BM + 4) + 4 * tx);
+    const float2 ah[2] = {make_float2(h.x, h.y), make_float2(h.z, h.w)};
+    const float2 al[2] = {make_float2(l.x, l.y), make_float2(l.z, l.w)};
+    const float2 nah[2] = {make_float2(-h.x, -h.y), make_float2(-h.z, -h.w)};
+#pragma unroll
+    for (int v = V0; v < U; ++v) {
+      const float4 q = Qs[kk * (BN + 1) + ty + 16 * v];
+      const float2 bh = make_float2(q.x, q.y), bl = make_float2(q.z, q.w);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) acc[u][v].add_prod(ah[u], nah[u], al[u], bh, bl);
+    }
+  }
+}
+
+template <int U, bool UPPER>
+__global__ void __launch_bounds__(256) k_gemm_nn_df(const double* __restrict__ A, long long lda,
+                                                    const double* __restrict__ Q, int ldq,
+                                                    long long d, int K, int n, double* C,
+                                                    long long ldc) {
+  constexpr int BM = 64, BN = 16 * U;
+  const long long r0 = (long long)blockIdx.x * BM;
+  const int j0 = blockIdx.y * BN;
+  __shared__ __align__(16) float Ah[GK * (BM + 4)], Al[GK * (BM + 4)];
+  __shared__ __align__(16) float4 Qs[GK * (BN + 1)];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  df64acc2 acc[2][U];
+  const int kend = UPPER ? min(K, j0 + BN) : K;
+  for (int k0 = 0; k0 < kend; k0 += GK) {
+#pragma unroll
+    for (int t = 0; t < GK * BM / 256; ++t) {
+      const int idx = tid + 256 * t, rr = idx % BM, kk = idx / BM;
+      const long long r = r0 + rr;
+      const df64 x((r < d && k0 + kk < K) ? A[r + (long long)(k0 + kk) * lda] : 0.0);
+      Ah[kk * (BM + 4) + rr] = x.hi;
+      Al[kk * (BM + 4) + rr] = x.lo;
+    }
+#pragma unroll
+    for (int t = 0; t < U; ++t) {
+      const int kk = tx, jj = ty + 16 * t;
+      const df64 x((k0 + kk < K && j0 + jj < n) ? Q[k0 + kk + (long long)(j0 + jj) * ldq] : 0.0);
+      Qs[kk * (BN + 1) + jj] = make_float4(x.hi, x.hi, x.lo, x.lo);
+    }
+    __syncthreads();
+    // first column group that rows k0 .. k0 + 15 of an upper triangular Q reach
+    switch (UPPER ? max(0, (k0 - j0) / 16) : 0) {
+      case 0: nn_df_step<U, 0>(Ah, Al, Qs, tx, ty, acc); break;
+      case 1: nn_df_step<U, (U > 1 ? 1 : U)>(Ah, Al, Qs, tx, ty, acc); break;
+      case 2: nn_df_step<U, (U > 2 ? 2 : U)>(Ah, Al, Qs, tx, ty, acc); break;
+      case 3: nn_df_step<U, (U > 3 ? 3 : U)>(Ah, Al, Qs, tx, ty, acc); break;
+      case 4: nn_df_step<U, (U > 4 ? 4 : U)>(Ah, Al, Qs, tx, ty, acc); break;
+      default: nn_df_step<U, (U > 5 ? 5 : U)>(Ah, Al, Qs, tx, ty, acc); break;
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int v = 0; v < U; ++v) {
+    const int j = j0 + ty + 16 * v;
+    if (j >= n) continue;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const long long r = r0 + 4 * tx + u;
+      if (r < d) C[r + (long long)j * ldc] = acc[u >> 1][v].value(u & 1).to_double();
+    }
+  }
+}
+
 template <typename F, typename Cm>
 static cudaError_t gemm_nn_impl(const F* A, long long lda, const F* Q, int ldq, long long d,
                                 int k, int n, double alpha, double beta, F* C, long long ldc,
-                                cudaStream_t stream) {
+                                cudaStream_t stream, bool upper) {
   const int u = tile_u(n);
   dim3 grid((unsigned)((d + 63) / 64), (n + 16 * u - 1) / (16 * u));
+#define CS_NN_CASE(UV)                                                                       \
+  case UV:                                                                                   \
+    if constexpr (std::is_same<Cm, df64>::value) {                                           \
+      if (upper)                                                                             \
+        k_gemm_nn_df<UV, true><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, C, ldc);   \
+      else                                                                                   \
+        k_gemm_nn_df<UV, false><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, C, ldc);  \
+    } else if (upper)                                                                               \
+      k_gemm_nn<F, Cm, UV, true><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, \
+                                                           (F)beta, C, ldc);                 \
+    else                                                                                     \
+      k_gemm_nn<F, Cm, UV, false><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, \
+                                                            (F)beta, C, ldc);                \
+    break;
   switch (u) {
-    case 1: k_gemm_nn<F, Cm, 1><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, (F)beta, C, ldc); break;
-    case 2: k_gemm_nn<F, Cm, 2><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, (F)beta, C, ldc); break;
-    case 3: k_gemm_nn<F, Cm, 3><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, (F)beta, C, ldc); break;
-    case 4: k_gemm_nn<F, Cm, 4><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, (F)beta, C, ldc); break;
-    case 5: k_gemm_nn<F, Cm, 5><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, (F)beta, C, ldc); break;
-    default: k_gemm_nn<F, Cm, 6><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, (F)beta, C, ldc); break;
+    CS_NN_CASE(1)
+    CS_NN_CASE(2)
+    CS_NN_CASE(3)
+    CS_NN_CASE(4)
+    CS_NN_CASE(5)
+    default:
+      CS_NN_CASE(6)
   }
+#undef CS_NN_CASE
   return cudaGetLastError();
 }
 
 template <typename F>
 cudaError_t launch_gemm_nn(const F* A, long long lda, const F* Q, int ldq, long long d, int k,
                            int n, double alpha, double beta, F* C, long long ldc,
-                           cudaStream_t stream) {
-  return gemm_nn_impl<F, F>(A, lda, Q, ldq, d, k, n, alpha, beta, C, ldc, stream);
+                           cudaStream_t stream, bool upper) {
+  return gemm_nn_impl<F, F>(A, lda, Q, ldq, d, k, n, alpha, beta, C, ldc, stream, upper);
 }
 
 cudaError_t launch_gemm_nn_df(const double* A, long long lda, const double* Q, int ldq,
                               long long d, int k, int n, double alpha, double beta, double* C,
-                              long long ldc, cudaStream_t stream) {
-  return gemm_nn_impl<double, df64>(A, lda, Q, ldq, d, k, n, alpha, beta, C, ldc, stream);
+                              long long ldc, cudaStream_t stream, bool upper) {
+  if (alpha != 1.0 || beta != 0.0) return cudaErrorInvalidValue;
+  return gemm_nn_impl<double, df64>(A, lda, Q, ldq, d, k, n, alpha, beta, C, ldc, stream, upper);
 }
 
 template cudaError_t launch_gram<double>(const double*, long long, const double*, long long,
@@ -248,10 +438,10 @@ template cudaError_t launch_gram<float>(const float*, long long, const float*, l
                                         long long, int, int, float*, int, float*, cudaStream_t);
 template cudaError_t launch_gemm_nn<double>(const double*, long long, const double*, int,
                                             long long, int, int, double, double, double*,
-                                            long long, cudaStream_t);
+                                            long long, cudaStream_t, bool);
 template cudaError_t launch_gemm_nn<float>(const float*, long long, const float*, int, long long,
                                            int, int, double, double, float*, long long,
-                                           cudaStream_t);
+                                           cudaStream_t, bool);
 
 // y[p + s ld] *= h[p]  (rows of an n_p x S block scaled by the projector couplings)
 template <typename F>
@@ -933,9 +1123,7 @@ __global__ void __launch_bounds__(1024) k_sym_eig(const double* __restrict__ Ain
 // All FP64 work here is wide (n x n GEMM tiles over many CTAs), which matters on a GPU
 // whose FP64 pipe is narrow: the FP32 factorisation carries the long serial chains.
 
-// C (n x n) = op(A) B, op(A) = A^T if TA; T x T output tiles, one element per thread. The FP64
-// pipe of one SM is narrow, so n <= 256 takes 8 x 8 tiles: at n = 80 that spreads the work over
-// 100 CTAs instead of 25 (16 x 16 tiles).
+// C (n x n) = op(A) B, op(A) = A^T if TA; T x T output tiles, one element per thread (n > 256).
 template <bool TA, int T>
 __global__ void __launch_bounds__(T * T) k_small_gemm(const double* __restrict__ A,
                                                        const double* __restrict__ B, int n,
@@ -957,12 +1145,47 @@ __global__ void __launch_bounds__(T * T) k_small_gemm(const double* __restrict__
   if (i < n && j < n) C[i + (size_t)j * n] = acc;
 }
 
+// n <= 256: up to two products in one launch (blockIdx.z), C[z] = op(A[z]) B[z]; 8 x 8 outputs per
+// CTA (at n = 80 over 100 CTAs: the FP64 pipe of one SM is narrow), the sum over k cut into four
+// ranges with two chains each, because a dependent FP64 multiply-add takes 64 cycles: 8 -> 4 us
+// at n = 80 against one chain per output.
+struct SmallGemm {
+  const double* A[2];
+  const double* B[2];
+  double* C[2];
+  int ta[2];
+};
+__global__ void __launch_bounds__(256) k_small_gemm_k4(SmallGemm g, int n) {
+  __shared__ double red[4][64];
+  const int z = blockIdx.z, t = threadIdx.x & 63, kg = threadIdx.x >> 6;
+  const int i = blockIdx.x * 8 + (t & 7), j = blockIdx.y * 8 + (t >> 3);
+  const double* __restrict__ A = g.A[z];
+  const double* __restrict__ B = g.B[z];
+  const int per = (n + 3) / 4, k1 = min(n, (kg + 1) * per);
+  double s0 = 0.0, s1 = 0.0;
+  if (i < n && j < n) {
+    const size_t sk = g.ta[z] ? 1 : n, si = g.ta[z] ? n : 1;
+    const double* a = A + si * i;
+    const double* b = B + (size_t)j * n;
+    int k = kg * per;
+#pragma unroll 4
+    for (; k + 1 < k1; k += 2) {
+      s0 = fma(a[sk * k], b[k], s0);
+      s1 = fma(a[sk * (k + 1)], b[k + 1], s1);
+    }
+    if (k < k1) s0 = fma(a[sk * k], b[k], s0);
+  }
+  red[kg][t] = s0 + s1;
+  __syncthreads();
+  if (kg == 0 && i < n && j < n)
+    g.C[z][i + (size_t)j * n] = (red[0][t] + red[1][t]) + (red[2][t] + red[3][t]);
+}
+
 static cudaError_t small_gemm(bool ta, const double* A, const double* B, int n, double* C,
                               cudaStream_t st) {
   if (n <= 256) {
-    dim3 grid((n + 7) / 8, (n + 7) / 8);
-    if (ta) k_small_gemm<true, 8><<<grid, 64, 0, st>>>(A, B, n, C);
-    else k_small_gemm<false, 8><<<grid, 64, 0, st>>>(A, B, n, C);
+    const SmallGemm g{{A, nullptr}, {B, nullptr}, {C, nullptr}, {ta, 0}};
+    k_small_gemm_k4<<<dim3((n + 7) / 8, (n + 7) / 8), 256, 0, st>>>(g, n);
   } else {
     dim3 grid((n + 15) / 16, (n + 15) / 16);
     if (ta) k_small_gemm<true, 16><<<grid, 256, 0, st>>>(A, B, n, C);
@@ -1002,15 +1225,17 @@ __global__ void __launch_bounds__(1024) k_oa_norms(const double* __restrict__ A,
     red[2][tid >> 5] = r2;
   }
   __syncthreads();
-  if (tid == 0) {
-    double ta = 0.0, ts = 0.0, tr = 0.0;
-    for (int w = 0; w < (nt + 31) / 32; ++w) {
-      ta += red[0][w];
-      ts += red[1][w];
-      tr += red[2][w];
+  if (tid < 32) {
+    double t[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      t[q] = tid < (nt + 31) / 32 ? red[q][tid] : 0.0;
+      for (int o = 16; o > 0; o >>= 1) t[q] += __shfl_xor_sync(0xffffffffu, t[q], o);
     }
-    scal[1] = sqrt(ta);
-    scal[0] = 2.0 * (sqrt(ts) + sqrt(ta) * sqrt(tr));
+    if (tid == 0) {
+      scal[1] = sqrt(t[0]);
+      scal[0] = 2.0 * (sqrt(t[1]) + sqrt(t[0]) * sqrt(t[2]));
+    }
   }
 }
 
@@ -1651,24 +1876,34 @@ cudaError_t launch_sym_eig(const double* A, int n, double* theta, double* V, dou
   };
   double* Vc = V0;
   double* Vn = V1;
-  for (int it = 0; it < 3; ++it) {
+  // FP32 vectors are orthonormal to 1e-6: two steps square that twice, below FP64's rounding
+  for (int it = 0; it < 2; ++it) {
     if ((e = prod(true, Vc, Vc, G)) != cudaSuccess) return e;   // G = V^T V
     k_ns_factor<<<(unsigned)((n2 + 255) / 256), 256, 0, stream>>>(G, n, Ep);
     if ((e = prod(false, Vc, Ep, Vn)) != cudaSuccess) return e;
     std::swap(Vc, Vn);
   }
+  // P = A V and G = V^T V (one launch for small n), S = V^T A V
+  auto project = [&]() -> cudaError_t {
+    cudaError_t r;
+    if (n <= 256) {
+      const SmallGemm g{{A, Vc}, {Vc, Vc}, {P, G}, {0, 1}};
+      k_small_gemm_k4<<<dim3((n + 7) / 8, (n + 7) / 8, 2), 256, 0, stream>>>(g, n);
+      r = cudaGetLastError();
+    } else {
+      if ((r = prod(false, A, Vc, P)) != cudaSuccess) return r;
+      r = prod(true, Vc, Vc, G);
+    }
+    return r == cudaSuccess ? prod(true, Vc, P, S) : r;
+  };
   for (int it = 0; it < 4; ++it) {
-    if ((e = prod(false, A, Vc, P)) != cudaSuccess) return e;   // P = A V
-    if ((e = prod(true, Vc, P, S)) != cudaSuccess) return e;    // S = V^T A V
-    if ((e = prod(true, Vc, Vc, G)) != cudaSuccess) return e;   // G = V^T V
+    if ((e = project()) != cudaSuccess) return e;
     oa_norms(A, S, G, lam, scal);
     k_oa_update<<<(unsigned)((n2 + 255) / 256), 256, 0, stream>>>(S, G, n, lam, scal, Ep);
     if ((e = prod(false, Vc, Ep, Vn)) != cudaSuccess) return e;  // V (I + E)
     std::swap(Vc, Vn);
   }
-  if ((e = prod(false, A, Vc, P)) != cudaSuccess) return e;
-  if ((e = prod(true, Vc, P, S)) != cudaSuccess) return e;
-  if ((e = prod(true, Vc, Vc, G)) != cudaSuccess) return e;
+  if ((e = project()) != cudaSuccess) return e;
   oa_norms(A, S, G, lam, scal);
   // 3. sort, clusters, output
   k_oa_final<<<1, 1024, 0, stream>>>(S, G, Vc, n, scal, theta, V, scratch, status);
@@ -1684,6 +1919,7 @@ __global__ void k_residuals(const double* __restrict__ X, long long ldx,
   const double* x = X + (size_t)col * ldx;
   const double* hx = HX + (size_t)col * ldh;
   double s = 0.0;
+#pragma unroll 4
   for (long long i = threadIdx.x; i < d; i += blockDim.x) {
     double r = hx[i] - th * x[i];
     s = fma(r, r, s);
@@ -1702,7 +1938,9 @@ __global__ void k_residuals(const double* __restrict__ X, long long ldx,
 cudaError_t launch_residuals(const double* X, long long ldx, const double* HX, long long ldh,
                              long long d, int n, const double* theta, double* resid,
                              cudaStream_t stream) {
-  k_residuals<<<n, 256, 0, stream>>>(X, ldx, HX, ldh, d, theta, resid);
+  // one CTA per column: 1024 threads, so that 80 columns keep enough loads in flight (87 us with
+  // 256 threads at d = 46128)
+  k_residuals<<<n, 1024, 0, stream>>>(X, ldx, HX, ldh, d, theta, resid);
   return cudaGetLastError();
 }
 
