@@ -13,10 +13,14 @@
 // States run in blocks of 32 (the three launches per block, one block-sized FA reused).
 // Exact identities only: the result differs from the row-pair and row-stream kernels by
 // rounding order.
+// The products run on packed FP32 instructions (df64acc2): two states per instruction. Shared
+// memory holds the states' leading and trailing parts apart, so that a pair is one register pair
+// as it is loaded.
 #include <cuda_runtime.h>
 
 #include <cstdint>
 #include <cstdlib>
+#include <type_traits>
 
 #include "cs_internal.h"
 #include "df64.cuh"
@@ -66,6 +70,28 @@ __host__ __device__ inline size_t df_l2_elems(const DfShape& s) {
 __host__ __device__ inline size_t df_p_elems(const DfShape& s) {
   return (size_t)4 * s.Qn * s.KC + (size_t)s.M2 * kDfSB + (size_t)4 * s.Qn * kDfSB + s.Np;
 }
+// the same with every trig value stored as both broadcast pairs
+__host__ __device__ inline size_t df_p_wide_elems(const DfShape& s) {
+  return df_p_elems(s) + (size_t)4 * s.Qn * s.KC;
+}
+
+// both broadcast pairs of a value
+__device__ __forceinline__ float4 df_bcast(df64 v) { return make_float4(v.hi, v.hi, v.lo, v.lo); }
+__device__ __forceinline__ float2 df_neg2(float2 v) { return make_float2(-v.x, -v.y); }
+// four states' parts as pairs
+struct DfQuad {
+  float2 h[2], n[2], l[2];
+  __device__ __forceinline__ DfQuad(const float* hi, const float* lo) {
+    const float4 a = *reinterpret_cast<const float4*>(hi);
+    const float4 b = *reinterpret_cast<const float4*>(lo);
+    h[0] = make_float2(a.x, a.y);
+    h[1] = make_float2(a.z, a.w);
+    l[0] = make_float2(b.x, b.y);
+    l[1] = make_float2(b.z, b.w);
+    n[0] = df_neg2(h[0]);
+    n[1] = df_neg2(h[1]);
+  }
+};
 
 struct DfArgs {
   int L, n_r, Nt, Np, S, s0, nmr;
@@ -102,7 +128,8 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_synth_df(DfArgs a) {
   const int r = blockIdx.x % a.nmr, k = blockIdx.x / a.nmr;
   const int it0 = (int)((long long)r * M2 / a.nmr), it1 = (int)((long long)(r + 1) * M2 / a.nmr);
   df64* th = reinterpret_cast<df64*>(smem_raw);   // [par][NP][KL]
-  df64* gs = th + (size_t)2 * NP * KL;            // [par][KL][SB]
+  float* gh = reinterpret_cast<float*>(th + (size_t)2 * NP * KL);  // [par][KL][SB], then lo
+  float* gl = gh + (size_t)2 * KL * kDfSB;
   df64* base = a.FA + (size_t)k * Nt * M2 * kDfSB;
   // tile: 2 pairs x 4 states, both parities
   const int ntile = ((NP + 1) / 2) * (kDfSB / 4);
@@ -116,13 +143,15 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_synth_df(DfArgs a) {
       const int par = idx / (KL * kDfSB), rem = idx - par * KL * kDfSB;
       const int i = rem / kDfSB, s = rem - i * kDfSB;
       const int l = am + par + 2 * i;
-      gs[idx] = (l <= lmax && s < ns) ? a.G[((size_t)k * L2 + l * l + l + m) * S + a.s0 + s]
-                                      : df64(0.f, 0.f);
+      const df64 g = (l <= lmax && s < ns) ? a.G[((size_t)k * L2 + l * l + l + m) * S + a.s0 + s]
+                                           : df64(0.f, 0.f);
+      gh[idx] = g.hi;
+      gl[idx] = g.lo;
     }
     __syncthreads();
     for (int ti = threadIdx.x; ti < ntile; ti += blockDim.x) {
       const int t0 = 2 * (ti / (kDfSB / 4)), s0 = 4 * (ti % (kDfSB / 4));
-      df64acc e[2][4], o[2][4];
+      df64acc2 e[2][2], o[2][2];
       const int t1 = min(t0 + 1, NP - 1);
       const df64* te0 = th + (size_t)t0 * KL;
       const df64* te1 = th + (size_t)t1 * KL;
@@ -130,20 +159,19 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_synth_df(DfArgs a) {
       const df64* to1 = te1 + (size_t)NP * KL;
       for (int i = 0; i < KL; ++i) {
         const df64 ae[2] = {te0[i], te1[i]}, ao[2] = {to0[i], to1[i]};
-        const float4* ge = reinterpret_cast<const float4*>(gs + (size_t)i * kDfSB + s0);
-        const float4* go = reinterpret_cast<const float4*>(gs + (size_t)(KL + i) * kDfSB + s0);
-        const float4 g0 = ge[0], g1 = ge[1], h0 = go[0], h1 = go[1];
-        const df64 be[4] = {df64(g0.x, g0.y), df64(g0.z, g0.w), df64(g1.x, g1.y),
-                            df64(g1.z, g1.w)};
-        const df64 bo[4] = {df64(h0.x, h0.y), df64(h0.z, h0.w), df64(h1.x, h1.y),
-                            df64(h1.z, h1.w)};
+        const DfQuad be(gh + i * kDfSB + s0, gl + i * kDfSB + s0);
+        const DfQuad bo(gh + (KL + i) * kDfSB + s0, gl + (KL + i) * kDfSB + s0);
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+        for (int u = 0; u < 2; ++u) {
+          const float4 x = df_bcast(ae[u]), y = df_bcast(ao[u]);
 #pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            e[u][v].add_prod(ae[u], be[v]);
-            o[u][v].add_prod(ao[u], bo[v]);
+          for (int v = 0; v < 2; ++v) {
+            e[u][v].add_prod_nb(make_float2(x.x, x.y), make_float2(x.z, x.w), be.h[v], be.n[v],
+                                be.l[v]);
+            o[u][v].add_prod_nb(make_float2(y.x, y.y), make_float2(y.z, y.w), bo.h[v], bo.n[v],
+                                bo.l[v]);
           }
+        }
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
@@ -154,7 +182,7 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_synth_df(DfArgs a) {
         df64* fb = base + ((size_t)tb * M2 + kap) * kDfSB + s0;
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          const df64 ev = e[u][v].value(), ov = o[u][v].value();
+          const df64 ev = e[u][v >> 1].value(v & 1), ov = o[u][v >> 1].value(v & 1);
           ft[v] = ev + ov;
           if (tb != t) fb[v] = ev - ov;
         }
@@ -164,15 +192,24 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_synth_df(DfArgs a) {
 }
 
 // ------------------------------------------------------------------------------------- P
+// WIDE: the trig table as float4 (both broadcast pairs); else as df64, where that does not fit
+template <bool WIDE>
 __global__ void __launch_bounds__(kDfThreads) k_phi_df(DfArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  using Tab = typename std::conditional<WIDE, float4, df64>::type;
   const DfShape sh = df_shape(a.L, a.Nt, a.Np);
   const int lmax = sh.lmax, M2 = sh.M2, Qn = sh.Qn, Q = sh.Q, KC = sh.KC;
   const int Nt = a.Nt, Np = a.Np, L = sh.L;
-  df64* tt = reinterpret_cast<df64*>(smem_raw);  // [c][q][i]
-  df64* fs = tt + (size_t)4 * Qn * KC;           // [kap][SB]
-  df64* hs = fs + (size_t)M2 * kDfSB;            // [c][q][SB]
-  df64* ws = hs + (size_t)4 * Qn * kDfSB;        // [p]
+  Tab* tt = reinterpret_cast<Tab*>(smem_raw);                        // [c][q][i]
+  float* fh = reinterpret_cast<float*>(tt + (size_t)4 * Qn * KC);    // [kap][SB], then lo
+  float* fl = fh + (size_t)M2 * kDfSB;
+  float* hh = fl + (size_t)M2 * kDfSB;                               // [c][q][SB], then lo
+  float* hl = hh + (size_t)4 * Qn * kDfSB;
+  df64* ws = reinterpret_cast<df64*>(hl + (size_t)4 * Qn * kDfSB);   // [p]
+  auto tab = [&](size_t i) -> float4 {
+    if constexpr (WIDE) return tt[i];
+    else return df_bcast(tt[i]);
+  };
   // class trig tables at the quarter angles, once per CTA
   for (int idx = threadIdx.x; idx < 4 * Qn * KC; idx += blockDim.x) {
     const int c = idx / (Qn * KC), rem = idx - c * Qn * KC;
@@ -180,7 +217,8 @@ __global__ void __launch_bounds__(kDfThreads) k_phi_df(DfArgs a) {
     const int mm = df_class_m(c, i);
     df64 v(0.f, 0.f);
     if (mm <= lmax) v = a.trig[((size_t)(c < 2 ? 0 : L) + mm) * Qn + q];
-    tt[idx] = v;
+    if constexpr (WIDE) tt[idx] = df_bcast(v);
+    else tt[idx] = v;
   }
   const long long ntiles = (long long)a.n_r * Nt;
   const int nsyn = ((Qn + 3) / 4) * (kDfSB / 2);   // synthesis tiles: 4 q x 2 states
@@ -192,15 +230,18 @@ __global__ void __launch_bounds__(kDfThreads) k_phi_df(DfArgs a) {
     __syncthreads();  // the previous tile is done with fs, hs, ws (and tt is complete)
     {
       const float4* src = reinterpret_cast<const float4*>(frow);
-      float4* dst = reinterpret_cast<float4*>(fs);
-      for (int idx = threadIdx.x; idx < M2 * kDfSB / 2; idx += blockDim.x) dst[idx] = src[idx];
+      for (int idx = threadIdx.x; idx < M2 * kDfSB / 2; idx += blockDim.x) {
+        const float4 f = src[idx];
+        reinterpret_cast<float2*>(fh)[idx] = make_float2(f.x, f.z);
+        reinterpret_cast<float2*>(fl)[idx] = make_float2(f.y, f.w);
+      }
       for (int idx = threadIdx.x; idx < Np; idx += blockDim.x) ws[idx] = wvr[idx];
     }
     __syncthreads();
     // class sums at 4 quarter angles x 2 states, folded with W V into the four classes
     for (int ti = threadIdx.x; ti < nsyn; ti += blockDim.x) {
       const int q0 = 4 * (ti / (kDfSB / 2)), s0 = 2 * (ti % (kDfSB / 2));
-      df64acc acc[4][4][2];
+      df64acc2 acc[4][4];
       int qq[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) qq[u] = min(q0 + u, Qn - 1);
@@ -209,14 +250,14 @@ __global__ void __launch_bounds__(kDfThreads) k_phi_df(DfArgs a) {
         for (int c = 0; c < 4; ++c) {
           const int kap = df_class_kap(c, i, lmax);
           if (kap < 0) continue;
-          const float4 f = *reinterpret_cast<const float4*>(fs + (size_t)kap * kDfSB + s0);
-          const df64 fv[2] = {df64(f.x, f.y), df64(f.z, f.w)};
-          const df64* tc = tt + (size_t)c * Qn * KC + i;
+          const float2 bh = *reinterpret_cast<const float2*>(fh + kap * kDfSB + s0);
+          const float2 bl = *reinterpret_cast<const float2*>(fl + kap * kDfSB + s0);
+          const float2 nbh = df_neg2(bh);
+          const size_t tc = (size_t)c * Qn * KC + i;
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const df64 tv = tc[(size_t)qq[u] * KC];
-            acc[c][u][0].add_prod(tv, fv[0]);
-            acc[c][u][1].add_prod(tv, fv[1]);
+            const float4 tv = tab(tc + (size_t)qq[u] * KC);
+            acc[c][u].add_prod_nb(make_float2(tv.x, tv.y), make_float2(tv.z, tv.w), bh, nbh, bl);
           }
         }
       }
@@ -228,8 +269,8 @@ __global__ void __launch_bounds__(kDfThreads) k_phi_df(DfArgs a) {
                    w4 = ws[(4 * Q - q) % Np];
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
-          const df64 ce = acc[0][u][v].value(), co = acc[1][u][v].value();
-          const df64 se = acc[2][u][v].value(), so = acc[3][u][v].value();
+          const df64 ce = acc[0][u].value(v), co = acc[1][u].value(v);
+          const df64 se = acc[2][u].value(v), so = acc[3][u].value(v);
           const df64 cp = ce + co, cm = ce - co, sp = se + so, sm = se - so;
           const df64 zero(0.f, 0.f);
           const df64 g1 = w1 * (cp + sp);
@@ -237,10 +278,13 @@ __global__ void __launch_bounds__(kDfThreads) k_phi_df(DfArgs a) {
           const df64 g3 = (q != 0) ? w3 * (cm + sm) : zero;
           const df64 g4 = (q != 0 && q != Q) ? w4 * (cp - sp) : zero;
           const int s = s0 + v;
-          hs[((size_t)0 * Qn + q) * kDfSB + s] = (g1 + g2) + (g3 + g4);
-          hs[((size_t)1 * Qn + q) * kDfSB + s] = (g1 - g2) - (g3 - g4);
-          hs[((size_t)2 * Qn + q) * kDfSB + s] = (g1 - g2) + (g3 - g4);
-          hs[((size_t)3 * Qn + q) * kDfSB + s] = (g1 + g2) - (g3 + g4);
+          const df64 r[4] = {(g1 + g2) + (g3 + g4), (g1 - g2) - (g3 - g4),
+                             (g1 - g2) + (g3 - g4), (g1 + g2) - (g3 + g4)};
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            hh[(c * Qn + q) * kDfSB + s] = r[c].hi;
+            hl[(c * Qn + q) * kDfSB + s] = r[c].lo;
+          }
         }
       }
     }
@@ -253,20 +297,18 @@ __global__ void __launch_bounds__(kDfThreads) k_phi_df(DfArgs a) {
       int ii[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) ii[u] = min(i0 + u, KC - 1);
-      df64acc acc[4][4];
-      const df64* tc = tt + (size_t)c * Qn * KC;
-      const df64* hc = hs + (size_t)c * Qn * kDfSB + s0;
+      df64acc2 acc[4][2];
       for (int q = 0; q < Qn; ++q) {
-        const df64* tq = tc + (size_t)q * KC;
-        const df64 tv[4] = {tq[ii[0]], tq[ii[1]], tq[ii[2]], tq[ii[3]]};
-        const float4* hp = reinterpret_cast<const float4*>(hc + (size_t)q * kDfSB);
-        const float4 h0 = hp[0], h1 = hp[1];
-        const df64 hv[4] = {df64(h0.x, h0.y), df64(h0.z, h0.w), df64(h1.x, h1.y),
-                            df64(h1.z, h1.w)};
+        const size_t tq = ((size_t)c * Qn + q) * KC;
+        const DfQuad hv(hh + (c * Qn + q) * kDfSB + s0, hl + (c * Qn + q) * kDfSB + s0);
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 4; ++u) {
+          const float4 tv = tab(tq + ii[u]);
 #pragma unroll
-          for (int v = 0; v < 4; ++v) acc[u][v].add_prod(tv[u], hv[v]);
+          for (int v = 0; v < 2; ++v)
+            acc[u][v].add_prod_nb(make_float2(tv.x, tv.y), make_float2(tv.z, tv.w), hv.h[v],
+                                  hv.n[v], hv.l[v]);
+        }
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -276,7 +318,7 @@ __global__ void __launch_bounds__(kDfThreads) k_phi_df(DfArgs a) {
         if (kap < 0) continue;
         df64* dst = frow + (size_t)kap * kDfSB + s0;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) dst[v] = acc[u][v].value();
+        for (int v = 0; v < 4; ++v) dst[v] = acc[u][v >> 1].value(v & 1);
       }
     }
   }
@@ -291,7 +333,8 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_anal_df(DfArgs a) {
   const int r = blockIdx.x % a.nmr, k = blockIdx.x / a.nmr;
   const int it0 = (int)((long long)r * M2 / a.nmr), it1 = (int)((long long)(r + 1) * M2 / a.nmr);
   df64* th = reinterpret_cast<df64*>(smem_raw);   // [par][NP][KL]
-  df64* ap = th + (size_t)2 * NP * KL;            // [par][NP][SB]
+  float* ph = reinterpret_cast<float*>(th + (size_t)2 * NP * KL);  // AP: [par][NP][SB], then lo
+  float* pl = ph + (size_t)2 * NP * kDfSB;
   const df64* base = a.FA + (size_t)k * Nt * M2 * kDfSB;
   const int per_par = ((KL + 1) / 2) * (kDfSB / 4);  // tiles: 2 l x 4 states per parity
   int cur_a = -1;
@@ -305,8 +348,11 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_anal_df(DfArgs a) {
       const int t = idx / kDfSB, s = idx - t * kDfSB, tb = Nt - 1 - t;
       const df64 x = base[((size_t)t * M2 + kap) * kDfSB + s];
       const df64 y = (tb != t) ? base[((size_t)tb * M2 + kap) * kDfSB + s] : df64(0.f, 0.f);
-      ap[idx] = x + y;
-      ap[(size_t)NP * kDfSB + idx] = (tb != t) ? x - y : df64(0.f, 0.f);
+      const df64 p = x + y, q = (tb != t) ? x - y : df64(0.f, 0.f);
+      ph[idx] = p.hi;
+      pl[idx] = p.lo;
+      ph[NP * kDfSB + idx] = q.hi;
+      pl[NP * kDfSB + idx] = q.lo;
     }
     __syncthreads();
     for (int ti = threadIdx.x; ti < 2 * per_par; ti += blockDim.x) {
@@ -314,18 +360,18 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_anal_df(DfArgs a) {
       const int i0 = 2 * (rem / (kDfSB / 4)), s0 = 4 * (rem % (kDfSB / 4));
       const int i1 = min(i0 + 1, KL - 1);
       const df64* tp = th + (size_t)par * NP * KL;
-      const df64* apb = ap + (size_t)par * NP * kDfSB + s0;
-      df64acc acc[2][4];
+      df64acc2 acc[2][2];
       for (int t = 0; t < NP; ++t) {
         const df64 tv[2] = {tp[(size_t)t * KL + i0], tp[(size_t)t * KL + i1]};
-        const float4* p = reinterpret_cast<const float4*>(apb + (size_t)t * kDfSB);
-        const float4 h0 = p[0], h1 = p[1];
-        const df64 hv[4] = {df64(h0.x, h0.y), df64(h0.z, h0.w), df64(h1.x, h1.y),
-                            df64(h1.z, h1.w)};
+        const DfQuad hv(ph + (par * NP + t) * kDfSB + s0, pl + (par * NP + t) * kDfSB + s0);
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+        for (int u = 0; u < 2; ++u) {
+          const float4 x = df_bcast(tv[u]);
 #pragma unroll
-          for (int v = 0; v < 4; ++v) acc[u][v].add_prod(tv[u], hv[v]);
+          for (int v = 0; v < 2; ++v)
+            acc[u][v].add_prod_nb(make_float2(x.x, x.y), make_float2(x.z, x.w), hv.h[v], hv.n[v],
+                                  hv.l[v]);
+        }
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
@@ -334,7 +380,8 @@ __global__ void __launch_bounds__(kDfThreads) k_leg_anal_df(DfArgs a) {
 #pragma unroll
         for (int v = 0; v < 4; ++v)
           if (s0 + v < ns)
-            a.G[((size_t)k * L2 + l * l + l + m) * S + a.s0 + s0 + v] = acc[u][v].value();
+            a.G[((size_t)k * L2 + l * l + l + m) * S + a.s0 + s0 + v] =
+                acc[u][v >> 1].value(v & 1);
       }
     }
   }
@@ -372,11 +419,13 @@ cudaError_t launch_angular_wide_df(const AngArgs<df64>& a, df64* G, df64* FA,
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return e;
   const size_t b1 = df_l1_elems(s) * sizeof(df64), b2 = df_l2_elems(s) * sizeof(df64);
-  const size_t bp = df_p_elems(s) * sizeof(df64);
+  const bool wide = df_p_wide_elems(s) * sizeof(df64) <= 227 * 1024;
+  const size_t bp = (wide ? df_p_wide_elems(s) : df_p_elems(s)) * sizeof(df64);
+  const auto phi = wide ? k_phi_df<true> : k_phi_df<false>;
   if ((e = cudaFuncSetAttribute(k_leg_synth_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)b1)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(k_phi_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)bp)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(phi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp)) !=
+          cudaSuccess ||
       (e = cudaFuncSetAttribute(k_leg_anal_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)b2)) != cudaSuccess)
     return e;
@@ -404,7 +453,7 @@ cudaError_t launch_angular_wide_df(const AngArgs<df64>& a, df64* G, df64* FA,
   for (int s0 = 0; s0 < a.S; s0 += kDfSB) {
     w.s0 = s0;
     k_leg_synth_df<<<a.n_r * nmr, kDfThreads, b1, stream>>>(w);
-    k_phi_df<<<(int)pgrid, kDfThreads, bp, stream>>>(w);
+    phi<<<(int)pgrid, kDfThreads, bp, stream>>>(w);
     k_leg_anal_df<<<a.n_r * nmr, kDfThreads, b2, stream>>>(w);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

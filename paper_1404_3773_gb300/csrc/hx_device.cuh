@@ -78,6 +78,27 @@ __device__ __forceinline__ void radial_synth_tile(const T* __restrict__ X, long 
   }
 }
 
+// The epilogue of one analysed coefficient z at row a of state s (see Epilogue)
+template <typename T>
+__device__ __forceinline__ void radial_epilogue(const Epilogue<T>& ep, size_t a, int s, T z) {
+  const size_t o = a + (size_t)s * ep.ld_out;
+  if (ep.mode == EP_PLAIN) {
+    ep.out[o] = z;
+    return;
+  }
+  const T x = ep.X[a + (size_t)s * ep.ld];
+  T hx = ep.half_lambda[a] * x + z;
+  if (ep.kb) hx += ep.kb[a + (size_t)s * ep.kb_ld];
+  if (ep.src) hx += ep.src_w[s] * ep.src[a + (size_t)s * ep.src_ld];
+  if (ep.mode == EP_APPLY) {
+    ep.out[o] = hx;
+  } else {  // EP_CHEB: out = cA (HX - c X) - cB Yprev   (out may alias Yprev)
+    T y = ep.cA * (hx - ep.cshift * x);
+    if (ep.Yprev) y -= ep.cB * ep.Yprev[o];
+    ep.out[o] = y;
+  }
+}
+
 // Z[alpha(l, mi, n), s] = sum_k rad[l][k][n] G[k][l^2 + mi][s], then the epilogue.
 template <typename T>
 __device__ __forceinline__ void radial_anal_tile(const T* __restrict__ G,
@@ -126,24 +147,7 @@ __device__ __forceinline__ void radial_anal_tile(const T* __restrict__ G,
     for (int i = 0; i < 4; ++i) {
       int n = nb0 + tx + 16 * i;
       if (n >= N) continue;
-      size_t a = (size_t)(l * l + mi) * N + n;
-      size_t o = a + (size_t)s * ep.ld_out;
-      T z = acc[i][j].value();
-      if (ep.mode == EP_PLAIN) {
-        ep.out[o] = z;
-        continue;
-      }
-      T x = ep.X[a + (size_t)s * ep.ld];
-      T hx = ep.half_lambda[a] * x + z;
-      if (ep.kb) hx += ep.kb[a + (size_t)s * ep.kb_ld];
-      if (ep.src) hx += ep.src_w[s] * ep.src[a + (size_t)s * ep.src_ld];
-      if (ep.mode == EP_APPLY) {
-        ep.out[o] = hx;
-      } else {  // EP_CHEB: out = cA (HX - c X) - cB Yprev   (out may alias Yprev)
-        T y = ep.cA * (hx - ep.cshift * x);
-        if (ep.Yprev) y -= ep.cB * ep.Yprev[o];
-        ep.out[o] = y;
-      }
+      radial_epilogue(ep, (size_t)(l * l + mi) * N + n, s, acc[i][j].value());
     }
   }
 }

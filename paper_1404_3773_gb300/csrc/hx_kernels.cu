@@ -48,6 +48,86 @@ __global__ void __launch_bounds__(256) k_radial_anal(const T* __restrict__ G,
   radial_anal_tile<T>(G, rad, L, N, n_r, S, ep, l, c0, blockIdx.y * RBM, As, Bs);
 }
 
+// Double-float: the 64 x 64 tiles of hx_device.cuh on packed FP32 instructions (df64acc2). A thread
+// owns 4 consecutive table rows (two operand pairs) x 4 columns; a column's value is stored as both
+// broadcast pairs. The same sums in the same order as the scalar tiles.
+template <int MODE>
+__global__ void __launch_bounds__(256) k_radial_df(const df64* __restrict__ X, long long ld,
+                                                    df64* __restrict__ G,
+                                                    const df64* __restrict__ rad, int L, int N,
+                                                    int n_r, int S, Epilogue<df64> ep) {
+  constexpr int PA = RBM + 4;
+  __shared__ __align__(16) float Ah[RBK * PA], Al[RBK * PA];
+  __shared__ __align__(16) float4 Bs[RBK][RBN + 1];
+  int l, c0;
+  locate_l_tile(blockIdx.x, S, l, c0);
+  const int m0 = blockIdx.y * RBM;  // first table row: radial node (0) or radial function (1)
+  const int ncol = (2 * l + 1) * S, L2 = L * L;
+  const int K = MODE == 0 ? N : n_r, M = MODE == 0 ? n_r : N;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int rg = MODE == 0 ? ty : tx, cg = MODE == 0 ? tx : ty;  // row and column groups
+  const df64* radl = rad + (size_t)l * n_r * N;
+  df64acc2 acc[2][4];
+  for (int q0 = 0; q0 < K; q0 += RBK) {
+    for (int idx = tid; idx < RBM * RBK; idx += 256) {
+      // consecutive threads along the table's contiguous index n
+      const int kk = MODE == 0 ? idx % RBK : idx / RBM, mm = MODE == 0 ? idx / RBK : idx % RBM;
+      const int q = q0 + kk, m = m0 + mm;
+      df64 v(0.f, 0.f);
+      if (m < M && q < K) v = MODE == 0 ? radl[(size_t)m * N + q] : radl[(size_t)q * N + m];
+      Ah[kk * PA + mm] = v.hi;
+      Al[kk * PA + mm] = v.lo;
+    }
+    for (int idx = tid; idx < RBN * RBK; idx += 256) {
+      const int kk = MODE == 0 ? idx % RBK : idx / RBN, cc = MODE == 0 ? idx / RBK : idx % RBN;
+      const int c = c0 + cc, q = q0 + kk;
+      df64 v(0.f, 0.f);
+      if (c < ncol && q < K) {
+        if (MODE == 0) {
+          const int mi = c / S, s = c - mi * S;
+          v = X[(size_t)(l * l + mi) * N + q + (size_t)s * ld];
+        } else {
+          v = G[((size_t)q * L2 + l * l) * S + c];
+        }
+      }
+      Bs[kk][cc] = make_float4(v.hi, v.hi, v.lo, v.lo);
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int kk = 0; kk < RBK; ++kk) {
+      const float4 h = *reinterpret_cast<const float4*>(Ah + kk * PA + 4 * rg);
+      const float4 w = *reinterpret_cast<const float4*>(Al + kk * PA + 4 * rg);
+      const float2 ah[2] = {make_float2(h.x, h.y), make_float2(h.z, h.w)};
+      const float2 al[2] = {make_float2(w.x, w.y), make_float2(w.z, w.w)};
+      const float2 nah[2] = {make_float2(-h.x, -h.y), make_float2(-h.z, -h.w)};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 b = Bs[kk][cg + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          acc[i][j].add_prod(ah[i], nah[i], al[i], make_float2(b.x, b.y), make_float2(b.z, b.w));
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = c0 + cg + 16 * j;
+    if (c >= ncol) continue;
+    const int mi = c / S, s = c - mi * S;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int m = m0 + 4 * rg + i;
+      if (m >= M) continue;
+      const df64 z = acc[i >> 1][j].value(i & 1);
+      if (MODE == 0)
+        G[((size_t)m * L2 + l * l) * S + c] = z;
+      else
+        radial_epilogue(ep, (size_t)(l * l + mi) * N + m, s, z);
+    }
+  }
+}
+
 // FP32: register-blocked tiles (radial_gemm.cuh), RM rows per thread chosen from M
 template <int MODE, int RM>
 __global__ void __launch_bounds__(kRgThreads) k_radial_gemm(const float* __restrict__ X,
@@ -370,6 +450,10 @@ cudaError_t launch_radial_synth(const T* X, long long ld, T* G, const T* rad, in
   if constexpr (std::is_same<T, float>::value)
     return launch_radial_gemm<0>(X, ld, G, rad, L, N, n_r, S, Epilogue<float>(), stream);
   dim3 grid(radial_col_tiles(L, S), (n_r + RBM - 1) / RBM);
+  if constexpr (std::is_same<T, df64>::value) {
+    k_radial_df<0><<<grid, 256, 0, stream>>>(X, ld, G, rad, L, N, n_r, S, Epilogue<df64>());
+    return cudaGetLastError();
+  }
   k_radial_synth<T><<<grid, 256, 0, stream>>>(X, ld, G, rad, L, N, n_r, S);
   return cudaGetLastError();
 }
@@ -380,6 +464,11 @@ cudaError_t launch_radial_anal(const T* G, const T* rad, int L, int N, int n_r, 
   if constexpr (std::is_same<T, float>::value)
     return launch_radial_gemm<1>(nullptr, 0, const_cast<float*>(G), rad, L, N, n_r, S, ep, stream);
   dim3 grid(radial_col_tiles(L, S), (N + RBM - 1) / RBM);
+  if constexpr (std::is_same<T, df64>::value) {
+    k_radial_df<1><<<grid, 256, 0, stream>>>(nullptr, 0, const_cast<df64*>(G), rad, L, N, n_r, S,
+                                             ep);
+    return cudaGetLastError();
+  }
   k_radial_anal<T><<<grid, 256, 0, stream>>>(G, rad, L, N, n_r, S, ep);
   return cudaGetLastError();
 }
