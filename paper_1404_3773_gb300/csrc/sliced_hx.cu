@@ -23,9 +23,11 @@
 //   R2  Z = sum_k R_ln(r_k) G', with the epilogue of the H.X and the Chebyshev recurrence
 // L1 .. L2 run over chunks of radial nodes so that the intermediates stay in the workspace slot.
 //
-// The kernels are bound by the integer pipe work of splitting (about 25 instructions per value)
-// and joining (about 30): the tensor cores are idle most of the time. Two CTAs of 256 threads
-// run per SM, so one CTA's loads and drains cover the other's waits. A thread owns the same
+// The kernels are bound by the instructions of splitting (about 40 per value with its load) and
+// joining (about 25): 0.75 G warp instructions for 80 states at lmax 30, issued at 35 % (radial) to
+// 60 % of the peak rate; the tensor cores are idle most of the time. That H.X takes 1.51 ms against
+// 7.13 on the FP64 pipe (whose peak would need 2.9 ms) and 2.41 in double-float. Two to four CTAs
+// of 256 threads run per SM, so one CTA's loads and drains cover the others' waits. A thread owns the same
 // operand row when it loads and when it drains, so its row's scale never leaves its registers.
 // Every mbarrier wait is bounded: on expiry the kernel records an error code in *err, frees its
 // tensor memory and returns.
@@ -57,8 +59,19 @@ constexpr int kRows = 128;     // operand rows per tile (MMA M)
 constexpr int kFix = 54;       // |value| <= 2^E is held as an integer in units of 2^(E - 54)
 constexpr int kADigit = kRows / 8 * 256;           // bytes of one (K step, digit): 4 KB
 constexpr int kBig = 1 << 20;
+constexpr int kNoUnit = (int)0x80808080;  // below every unit (a memset of 0x80)
 
 enum { OP_R1, OP_L1, OP_P1, OP_P2, OP_L2, OP_R2 };
+
+// Programmatic dependent launch (SlPlan says when): a kernel of the chain lets the next one start its prologue
+// (barriers, tensor memory, table images) at once, and touches the chain's data only when the
+// kernel before it has completed and its writes are visible.
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // bytes of one table image: `ks` K steps, nb table rows
 __host__ __device__ inline size_t img_bytes(int ks, int nb) {
@@ -189,7 +202,9 @@ struct SlArgs {
   const int* shP;                   // P2: shift of W's row
   const int* uP;                    // unit of AP's row
   const int* U;                     // [k'][SB] largest uP of the node
+  int* Uw;                          // the same, to be written
   long long ntiles;
+  bool early;                       // host: launch with programmatic dependence
   int c4 = 1 << 4, c20 = 1 << 20;  // see join_diags
   int* err;
   Epilogue<double> ep;              // R2
@@ -337,9 +352,15 @@ __device__ __forceinline__ void sl_load8(const SlArgs& a, const SlRow& w, int cl
   }
 }
 
+// CTAs per SM: 16-column blocks take 128 of the 512 columns of tensor memory, and the syntheses
+// fit 64 registers; P2 and L2 hold K = 32 in shared memory (70 KB)
+constexpr int sl_ctas(int op, int nb) {
+  return nb != 16 ? 2 : (op == OP_L1 || op == OP_P1 ? 4 : 3);
+}
+
 // SMALL: at most 32 k per accumulation (join_diags)
 template <int OP, int NB, bool SMALL>
-__global__ void __launch_bounds__(kSlThreads, NB == 16 ? 3 : 2) k_sl(SlArgs a) {
+__global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar_b[2], bar_mma;
   __shared__ uint32_t tmem_base_sh;
@@ -366,6 +387,9 @@ __global__ void __launch_bounds__(kSlThreads, NB == 16 ? 3 : 2) k_sl(SlArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
+  // only now: a kernel further down the chain must not take the tensor memory that this one,
+  // which it waits for, still asks for
+  pdl_trigger();
   const uint32_t sA = smem_u32(smem), sB = sA + (uint32_t)(ksmax * kDig * kADigit);
   const uint32_t bslot = (uint32_t)(ksmax * kBStep);
 
@@ -391,6 +415,10 @@ __global__ void __launch_bounds__(kSlThreads, NB == 16 ? 3 : 2) k_sl(SlArgs a) {
   int table;
   sl_locate<OP>(a, t0, r, w, table);
   if (tid == 0 && t0 < t1) issue_b(table, 0, 0, 0);
+  pdl_wait();
+  if constexpr (OP == OP_L1)  // the units' maxima of the chunk start from nothing
+    for (int i = blockIdx.x * kSlThreads + tid; i < a.kc * a.SB; i += gridDim.x * kSlThreads)
+      a.Uw[i] = kNoUnit;
 
   bool ok = true;    // block-uniform
   bool good = true;  // this thread's waits
@@ -682,6 +710,8 @@ __global__ void __launch_bounds__(256) k_sl_pointwise(long long* __restrict__ W,
                                                       int* __restrict__ shP,
                                                       int* __restrict__ uP,
                                                       int* __restrict__ U) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int red[8][32];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const long long i = (long long)blockIdx.x * 32 + lane;
@@ -740,6 +770,8 @@ __global__ void __launch_bounds__(256) k_sl_fold(const double* __restrict__ g,
                                                  long long* __restrict__ W,
                                                  int* __restrict__ shP, int* __restrict__ uP,
                                                  int* __restrict__ U) {
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (i >= (long long)rows * SB) return;
@@ -798,6 +830,8 @@ __global__ void __launch_bounds__(256) k_sl_grid(const long long* __restrict__ W
                                                  const int* __restrict__ eW, int rows, int SB,
                                                  int s0, int k0, int Nt, int Np, int Q, int n_r,
                                                  double* __restrict__ f) {
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (i >= (long long)rows * SB) return;
@@ -829,6 +863,8 @@ __global__ void __launch_bounds__(256) k_sl_density(const long long* __restrict_
                                                     int Np, int Q, int k0,
                                                     const double* __restrict__ occ,
                                                     double* __restrict__ rho, int accumulate) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ double dsm[];  // [4 Q][33], then weights [32]
   double* wt = dsm + 4 * Q * 33;
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -885,6 +921,8 @@ __global__ void __launch_bounds__(256) k_sl_density(const long long* __restrict_
 // E_G[k][s]: 2^E above every |G[k][lm][s]|
 __global__ void __launch_bounds__(256) k_sl_gexp(const double* __restrict__ G, int L2, int S,
                                                  int* __restrict__ EG) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int red[8][32];
   const int s = blockIdx.x * 32 + (threadIdx.x & 31), k = blockIdx.y, wp = threadIdx.x >> 5;
   int mx = 0;
@@ -1054,6 +1092,22 @@ void chunking(int L, int n_r, int n_theta, int n_phi, int S, int& SB, int& kc) {
   kc = (n_r + nchunks - 1) / nchunks;
 }
 
+template <class... P, class... A>
+cudaError_t launch_chain(bool early, void (*kernel)(P...), unsigned grid_x, unsigned grid_y,
+                         int threads, int smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid_x, grid_y);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 template <int OP, int NB, bool SMALL>
 cudaError_t launch_sl(const SlArgs& a, const Geo& g, cudaStream_t st) {
   const int ks = g.nch > 1 ? 2 : g.lastks;
@@ -1065,9 +1119,9 @@ cudaError_t launch_sl(const SlArgs& a, const Geo& g, cudaStream_t st) {
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return e;
-  const unsigned grid = (unsigned)std::min<long long>(a.ntiles, (NB == 16 ? 3ll : 2ll) * nsm);
-  k_sl<OP, NB, SMALL><<<grid, kSlThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  const int fit = std::min(sl_ctas(OP, NB), 227 * 1024 / (smem + 3 * 1024));
+  const unsigned grid = (unsigned)std::min<long long>(a.ntiles, (long long)fit * nsm);
+  return launch_chain(a.early, k_sl<OP, NB, SMALL>, grid, 1, kSlThreads, smem, st, a);
 }
 // P2, L2: up to 16 or 32 modes per class, up to 32 or 64 k
 template <int OP>
@@ -1206,6 +1260,11 @@ struct SlPlan {
     a.M2 = 2 * L - 1;
     a.Q = Np / 4 + 1;
     a.S = S;
+    // An early launch hides a few microseconds per kernel, which counts in small problems: lmax 10,
+    // 16 states 88 -> 76 us, 64 states 129 -> 114. In larger ones the next kernel's CTAs take the
+    // room of the running one's unevenly: lmax 30, one state 221 -> 324 us; lmax 23, 4 states 160
+    // -> 167; the two meet near rows L^2 = 7M at lmax 16 (16 states: 130 us both).
+    a.early = L <= 17 && (long long)H.n_r * H.n_theta * S * L2 < 6000000;
     a.F1 = T.F1;
     a.ks = (half + 15) / 16;
     a.nb2 = half <= 16 ? 16 : 32;
@@ -1221,6 +1280,7 @@ struct SlPlan {
     a.shP = shP;
     a.uP = uP;
     a.U = U;
+    a.Uw = U;
     a.EG = EG;
     a.err = err;
   }
@@ -1244,9 +1304,8 @@ struct SlPlan {
     return launch_sl<OP_R2, 32, false>(a, g[OP_R2], st);
   }
   cudaError_t scales() {
-    k_sl_gexp<<<dim3((a.S + 31) / 32, H.n_r), 256, 0, st>>>(a.G, L2, a.S, EG);
     ++n;
-    return cudaGetLastError();
+    return launch_chain(a.early, k_sl_gexp, (a.S + 31) / 32, H.n_r, 256, 0, st, a.G, L2, a.S, EG);
   }
   void legendre_tiles() {
     const int nodes = a.kc * a.SB;
@@ -1316,13 +1375,12 @@ cudaError_t launch_sliced_hx(const HostTables& H, const SlicedTables& T, int S, 
   } else {
     SL_TRY(p.scales());
     e = p.chunks([&]() -> cudaError_t {
-      SL_TRY(p.clear_units());
       SL_TRY(p.synth());
       const int rows = p.rows();
-      k_sl_pointwise<<<(unsigned)(((long long)rows * a.SB + 31) / 32), 256, 0, st>>>(
-          a.W, a.eW, T.wv, T.ewv, rows, a.SB, a.Nt, p.Np, a.Q, a.k0, p.shP, p.uP, p.U);
       ++p.n;
-      SL_TRY(cudaGetLastError());
+      SL_TRY(launch_chain(a.early, k_sl_pointwise, (unsigned)(((long long)rows * a.SB + 31) / 32), 1, 256, 0,
+                        st, a.W, a.eW, T.wv, T.ewv, rows, a.SB, a.Nt, p.Np, a.Q, a.k0, p.shP, p.uP,
+                        p.U));
       return p.anal();
     });
   }
@@ -1340,10 +1398,9 @@ cudaError_t launch_sliced_grid(const HostTables& H, const SlicedTables& T, int S
   SL_TRY(p.chunks([&]() -> cudaError_t {
     SL_TRY(p.synth());
     const int rows = p.rows();
-    k_sl_grid<<<warp_grid((long long)rows * a.SB), 256, 0, st>>>(a.W, a.eW, rows, a.SB, a.s0, a.k0,
-                                                                 a.Nt, p.Np, a.Q, H.n_r, f);
     ++p.n;
-    return cudaGetLastError();
+    return launch_chain(a.early, k_sl_grid, warp_grid((long long)rows * a.SB), 1, 256, 0, st, a.W, a.eW, rows,
+                      a.SB, a.s0, a.k0, a.Nt, p.Np, a.Q, H.n_r, f);
   }));
   *launches = p.n;
   return cudaSuccess;
@@ -1361,10 +1418,9 @@ cudaError_t launch_sliced_density(const HostTables& H, const SlicedTables& T, in
   SL_TRY(cudaFuncSetAttribute(k_sl_density, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   SL_TRY(p.chunks([&]() -> cudaError_t {
     SL_TRY(p.synth());
-    k_sl_density<<<(unsigned)p.rows(), 256, smem, st>>>(a.W, a.eW, a.SB, a.Nt, p.Np, a.Q, a.k0,
-                                                       occ + a.s0, rho, add || a.s0 > 0 ? 1 : 0);
     ++p.n;
-    return cudaGetLastError();
+    return launch_chain(a.early, k_sl_density, (unsigned)p.rows(), 1, 256, smem, st, a.W, a.eW, a.SB, a.Nt,
+                      p.Np, a.Q, a.k0, occ + a.s0, rho, add || a.s0 > 0 ? 1 : 0);
   }));
   *launches = p.n;
   return cudaSuccess;
@@ -1379,10 +1435,9 @@ cudaError_t launch_sliced_forward(const HostTables& H, const SlicedTables& T, in
   SL_TRY(p.chunks([&]() -> cudaError_t {
     SL_TRY(p.clear_units());
     const int rows = p.rows();
-    k_sl_fold<<<warp_grid((long long)rows * a.SB), 256, 0, st>>>(
-        g, wkj, rows, a.SB, a.s0, a.k0, a.Nt, p.Np, a.Q, H.n_r, a.W, p.shP, p.uP, p.U);
     ++p.n;
-    SL_TRY(cudaGetLastError());
+    SL_TRY(launch_chain(a.early, k_sl_fold, warp_grid((long long)rows * a.SB), 1, 256, 0, st, g, wkj, rows,
+                      a.SB, a.s0, a.k0, a.Nt, p.Np, a.Q, H.n_r, a.W, p.shP, p.uP, p.U));
     return p.anal();
   }));
   SL_TRY(p.radial_anal(ep));
