@@ -226,31 +226,34 @@ __global__ void __launch_bounds__(kThreads) k_tc_radial(TcShape sh,
   // epilogue: warp w reads TMEM lanes 32w..32w+31 (the tile's columns), 16 radial rows per
   // load; thread = one column c
   const int c = c0 + warp * 32 + lane;
-  const bool live = ok && c < ncol;
   int mi = 0, s = 0;
   if (c < ncol) {
     mi = c / sh.S;
     s = c - mi * sh.S;
   }
-  // weight of the residual-form source term of this column (0 when there is none)
-  const float sw = (MODE == 1 && ep.src && c < ncol) ? ep.src_w[s] : 0.f;
-  if (ok) {
+  if (MODE == 0 && ok) {
     for (int rb = 0; rb < rows; rb += 16) {
       float v[16];
       tmem_ld16(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)rb, v);
-      if (!live) continue;
-      if (MODE == 0) {
-        // G[k][l^2 + mi][s] for k = rb .. rb + 15: lanes (consecutive c) write consecutive words
+      if (c >= ncol) continue;
+      // G[k][l^2 + mi][s] for k = rb .. rb + 15: lanes (consecutive c) write consecutive words
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int k = rb + i;
-          if (k < Mout) G[((size_t)k * L2 + l * l) * sh.S + c] = v[i];
-        }
-        continue;
+      for (int i = 0; i < 16; ++i) {
+        const int k = rb + i;
+        if (k < Mout) G[((size_t)k * L2 + l * l) * sh.S + c] = v[i];
       }
+    }
+  }
+  if (MODE == 1 && ok && vec_ep) {
+    // weight of the residual-form source term of this column (0 when there is none)
+    const float sw = (ep.src && c < ncol) ? ep.src_w[s] : 0.f;
+    for (int rb = 0; rb < rows; rb += 16) {
+      float v[16];
+      tmem_ld16(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)rb, v);
+      if (c >= ncol) continue;
       // Z[alpha(l, mi, n), s] for n = rb .. rb + 15 (contiguous in n)
       const size_t a0 = (size_t)(l * l + mi) * sh.N;
-      if (vec_ep && rb + 16 <= Mout) {
+      if (rb + 16 <= Mout) {
         // 16-byte runs: four float4 of each operand (a0 + rb, s ld, s ld_out multiples of 4)
         const size_t a = a0 + rb;
         const size_t o = a + (size_t)s * ep.ld_out;
@@ -326,6 +329,81 @@ __global__ void __launch_bounds__(kThreads) k_tc_radial(TcShape sh,
           float y = __fmul_rn(ep.cA, fmaf(-ep.cshift, x, hx));
           if (ep.Yprev) y = fmaf(-ep.cB, ep.Yprev[o], y);
           ep.out[o] = y;
+        }
+      }
+    }
+  }
+  if (MODE == 1 && ok && !vec_ep) {
+    // Z[alpha(l, mi, n), s] is contiguous in n, a thread's column is not contiguous with its
+    // neighbours': the tile goes through shared memory (the operand buffers, now free) so that
+    // the block, the recurrence term and the output are read and written along n, whatever their
+    // alignment: 43 -> 26 us at d = 24192, 53 states against one thread per column in single words.
+    // Where 16-byte runs are possible they stay (above): 31 us against 42 at d = 46128, 80 states.
+    float* Zs = reinterpret_cast<float*>(smem);
+    const int cap = (2 * (rows + TC) * KC * 2) / (TC * 4) - 1;  // rows per pass
+    const int rp = rows <= cap ? rows : cap & ~15;
+    const int zp = rp + 1;  // odd pitch: a warp's 32 columns start on different banks
+    __shared__ int col_a[TC], col_s[TC];
+    col_a[tid] = (l * l + mi) * sh.N;
+    col_s[tid] = s;
+    const int ncl = min(TC, ncol - c0);
+    for (int r0 = 0; r0 < Mout; r0 += rp) {
+      if (r0 > 0) __syncthreads();
+      for (int rb = 0; rb < rp && r0 + rb < rows; rb += 16) {
+        float v[16];
+        tmem_ld16(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)(r0 + rb), v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) Zs[tid * zp + rb + i] = v[i];
+      }
+      __syncthreads();
+      const int m = min(rp, Mout - r0), total = ncl * m;
+      const int dq = kThreads / m, dr = kThreads - dq * m;
+      int col = tid / m, n = tid - col * m;
+      constexpr int UB = 8;
+      for (int i0 = tid; i0 < total; i0 += UB * kThreads) {
+        // all loads of the batch before its stores (out may alias Yprev)
+        float z[UB], x[UB], h[UB], kb[UB], y[UB], sr[UB], sw[UB];
+        size_t o[UB];
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+          if (i0 + u * kThreads < total) {
+            const int st = col_s[col];
+            const size_t a = (size_t)col_a[col] + r0 + n;
+            o[u] = a + (size_t)st * ep.ld_out;
+            z[u] = Zs[col * zp + n];
+            if (ep.mode != EP_PLAIN) {
+              x[u] = ep.X[a + (size_t)st * ep.ld];
+              h[u] = ep.half_lambda[a];
+              kb[u] = ep.kb ? ep.kb[a + (size_t)st * ep.kb_ld] : 0.f;
+              y[u] = ep.Yprev && ep.mode == EP_CHEB ? ep.Yprev[o[u]] : 0.f;
+              sr[u] = ep.src ? ep.src[a + (size_t)st * ep.src_ld] : 0.f;
+              sw[u] = ep.src ? ep.src_w[st] : 0.f;
+            }
+          }
+          col += dq;
+          n += dr;
+          if (n >= m) {
+            n -= m;
+            ++col;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+          if (i0 + u * kThreads >= total) continue;
+          float r = z[u];
+          if (ep.mode != EP_PLAIN) {
+            // the same roundings as the FP32 radial tiles (fmaf, __fmul_rn, __fadd_rn)
+            float hx = fmaf(h[u], x[u], z[u]);
+            if (ep.kb) hx = __fadd_rn(hx, kb[u]);
+            if (ep.src) hx = fmaf(sw[u], sr[u], hx);
+            if (ep.mode == EP_APPLY) {
+              r = hx;
+            } else {
+              r = __fmul_rn(ep.cA, fmaf(-ep.cshift, x[u], hx));
+              if (ep.Yprev) r = fmaf(-ep.cB, y[u], r);
+            }
+          }
+          ep.out[o[u]] = r;
         }
       }
     }
