@@ -44,6 +44,7 @@ using namespace tcx;
 
 constexpr int kWaThreads = 256;
 constexpr int kPThreads = 512;  // the phi pass
+constexpr int kL2Threads = 256;  // the Legendre quadrature: four warps per parity
 constexpr int kWaRows = 128;  // MMA M: the states of one block
 constexpr int kSmemPerSM = 228 * 1024;
 
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(kWaThreads)
   const int ntask = kWaRows * 2 * (KL / 8);
   if (tid == 0) {
     mbar_init(bar_tab, 1);
-    mbar_init(bar_mma, 1);
+    mbar_init(bar_mma, 2);  // one commit per parity
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(smem_u32(&tmem_sh), tcols);
@@ -241,9 +242,12 @@ __global__ void __launch_bounds__(kWaThreads)
     }
     ok = __syncthreads_and(t_ok ? 1 : 0) != 0;
     if (!ok) break;
-    if (tid == 0) {
+    // each parity's MMAs from a warp of their own: the accumulators are apart, and one thread
+    // takes longer to issue both than the tensor cores to run them
+    if (lane == 0 && warp < 2) {
       tc_fence_after();
-      for (int par = 0; par < 2; ++par) {
+      {
+        const int par = warp;
         const uint32_t ah = smem_u32(sA + (size_t)par * 2 * aplane), al = ah + (uint32_t)aplane;
         const uint32_t bh = smem_u32(sB + (size_t)par * 2 * bplane), bl = bh + (uint32_t)bplane;
         for (int ks = 0; ks < KL / 16; ++ks) {
@@ -295,11 +299,12 @@ __global__ void __launch_bounds__(kWaThreads)
 }
 
 // ------------------------------------------------------------------------------------ L2
-// 512 threads. NT: operand tasks (8 pairs each) per thread and mode, an upper bound on NPp / 32;
-// the next
-// mode's AP values are loaded into registers while this mode's MMAs and stores run.
+// NT: operand tasks (8 pairs each) per thread and mode, an upper bound on NPp / 16; the next
+// mode's AP values are loaded into registers while this mode's MMAs and stores run. Two CTAs of
+// 256 threads per SM, so that one loads and splits while the other waits for its MMAs (one CTA
+// of 512: 0.71 ms at lmax 60, 128 states).
 template <int NT>
-__global__ void __launch_bounds__(kPThreads, 1)
+__global__ void __launch_bounds__(kL2Threads, 2)
     k_leg_anal_tc(WaArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[2];
@@ -320,7 +325,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
   const int ntask = kWaRows * (NPp / 8);
   if (tid == 0) {
     mbar_init(bar_tab, 1);
-    mbar_init(bar_mma, 1);
+    mbar_init(bar_mma, 2);  // one commit per parity
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(smem_u32(&tmem_sh), tcols);
@@ -337,7 +342,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const int kap = item_m(it) + lmax;
 #pragma unroll
     for (int u = 0; u < NT; ++u) {
-      const int task = tid + u * kPThreads;
+      const int task = tid + u * kL2Threads;
       const int s = task & (kWaRows - 1), tg = task >> 7;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
@@ -364,7 +369,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     // A[0][s][t] = AP(t) + AP(mirror t), A[1][s][t] = AP(t) - AP(mirror t)
 #pragma unroll
     for (int u = 0; u < NT; ++u) {
-      const int task = tid + u * kPThreads;
+      const int task = tid + u * kL2Threads;
       if (task < ntask) {
         const int s = task & (kWaRows - 1), tg = task >> 7;
         float e[8], o[8];
@@ -389,9 +394,12 @@ __global__ void __launch_bounds__(kPThreads, 1)
     }
     ok = __syncthreads_and(t_ok ? 1 : 0) != 0;
     if (!ok) break;
-    if (tid == 0) {
+    // each parity's MMAs from a warp of their own: the accumulators are apart, and one thread
+    // takes longer to issue both than the tensor cores to run them
+    if (lane == 0 && warp < 2) {
       tc_fence_after();
-      for (int par = 0; par < 2; ++par) {
+      {
+        const int par = warp;
         const uint32_t ah = smem_u32(sA + (size_t)par * 2 * aplane), al = ah + (uint32_t)aplane;
         const uint32_t uh = smem_u32(sU + (size_t)par * 2 * uplane), ul = uh + (uint32_t)uplane;
         for (int ks = 0; ks < NPp / 16; ++ks) {
@@ -412,11 +420,10 @@ __global__ void __launch_bounds__(kPThreads, 1)
     ok = __syncthreads_and(w_ok ? 1 : 0) != 0;
     if (!ok) break;
     tc_fence_after();
-    // G'[l = am + par + 2i, m][s]; warps 4..7 and 12..15 the odd parity, warps 8..15 every
-    // other 16 l
+    // G'[l = am + par + 2i, m][s]; warps 4..7 the odd parity
     {
-      const int qd = warp & 3, par = (warp >> 2) & 1, s = 32 * qd + lane;
-      for (int i0 = 16 * (warp >> 3); i0 < KL; i0 += 32) {
+      const int qd = warp & 3, par = warp >> 2, s = 32 * qd + lane;
+      for (int i0 = 0; i0 < KL; i0 += 16) {
         float v[16];
         tmem_ld16_issue(tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(par * KL + i0), v);
         tmem_ld_wait();
@@ -465,7 +472,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
   if (tid == 0) {
     mbar_init(bar_tab, 1);
     mbar_init(bar_f, 1);
-    mbar_init(bar_mma, 1);
+    mbar_init(bar_mma, 4);  // one commit per class
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(smem_u32(&tmem_sh), tcols);
@@ -526,7 +533,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
-    if (tid == 0) {
+    if (tid == 4 * 32) {
       const long long tn = tl + gridDim.x;
       if (tn < ntiles) {  // the F rows are consumed: stream the next tile's into them
         const float *f, *w;
@@ -535,8 +542,13 @@ __global__ void __launch_bounds__(kPThreads, 1)
         bulk_g2s(smem_u32(smem + ps.f), f, fbytes, bar_f);
         bulk_g2s(smem_u32(smem + ps.wv + (size_t)(buf ^ 1) * Np * 4), w, wbytes, bar_f);
       }
+    }
+    // each class's MMAs from a warp of their own: the accumulators are apart, and one thread
+    // takes longer to issue all 24 than the tensor cores to run them
+    if (lane == 0 && warp < 4) {
       tc_fence_after();
-      for (int c = 0; c < 4; ++c) {
+      {
+        const int c = warp;
         const uint32_t ah = smem_u32(sA + (size_t)c * 2 * fplane), al = ah + (uint32_t)fplane;
         const uint32_t bh = smem_u32(sT + (size_t)c * 2 * tplane), bl = bh + (uint32_t)tplane;
         for (int ks = 0; ks < KC / 16; ++ks) {
@@ -594,9 +606,10 @@ __global__ void __launch_bounds__(kPThreads, 1)
       fence_async_smem();
       tc_fence_before();
       __syncthreads();
-      if (tid == 0) {
+      if (lane == 0 && warp < 4) {
         tc_fence_after();
-        for (int c = 0; c < 4; ++c) {
+        {
+          const int c = warp;
           const uint32_t ah = smem_u32(sA + (size_t)c * 2 * hplane), al = ah + (uint32_t)hplane;
           const uint32_t uh = smem_u32(sUt + (size_t)c * 2 * tplane), ul = uh + (uint32_t)tplane;
           for (int ks = 0; ks < QH / 16; ++ks) {
@@ -789,11 +802,11 @@ cudaError_t launch_angular_wide(const AngArgs<float>& a, const void* tab, float*
   k_phi_tc<<<(int)grid, kPThreads, req, stream>>>(w);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   residency(l2_smem(s), pow2_cols(2 * s.KL), per_sm, req);
-  auto l2 = s.NPp <= 32 ? k_leg_anal_tc<1> : k_leg_anal_tc<2>;
+  auto l2 = s.NPp <= 32 ? k_leg_anal_tc<2> : k_leg_anal_tc<4>;
   if ((e = cudaFuncSetAttribute(l2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)req)) !=
       cudaSuccess)
     return e;
-  l2<<<base * nmr, kPThreads, req, stream>>>(w);
+  l2<<<base * nmr, kL2Threads, req, stream>>>(w);
   return cudaGetLastError();
 }
 
