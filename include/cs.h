@@ -67,7 +67,10 @@ typedef struct {
 } cs_quadrature;
 
 typedef enum {
-  CS_FP64 = 0,       /* FP64 storage and arithmetic                                      */
+  CS_FP64 = 0,       /* FP64 storage and accuracy: FP64 arithmetic, or, for blocks from 4096
+                        grid rows x states (N_r N_theta n_s), exact products of 8-bit integer
+                        slices on the tensor cores with 64-bit integer sums between them
+                        (agreement with the FP64 arithmetic to a few units of 2^-53)      */
   CS_FP32 = 1,       /* FP32 storage and arithmetic (FP32 FMA pipe)                      */
   CS_MIXED_BF16 = 2  /* FP32 storage; the per-l radial contractions on the tensor cores
                         (tcgen05) with operands split into two BF16 terms (hi + lo, three
@@ -79,8 +82,9 @@ typedef enum {
                         arithmetic on the FP32 pipe (each value an unevaluated sum of two
                         floats, about 48 significant bits; Dekker/Knuth error-free
                         transformations). On a GPU whose FP64 pipe runs at 1/64 of the FP32
-                        rate this is several times faster than CS_FP64 at relative errors
-                        near 1e-14. With projectors it is available for cs_apply_H and the
+                        rate this is faster than FP64 arithmetic at relative errors near 1e-14.
+                        Blocks with N_r N_theta n_s (lmax+1)^2 >= 14e6 take CS_FP64's slice
+                        products instead. With projectors it is available for cs_apply_H and the
                         Rayleigh-Ritz apply only, and only with CS_FP64_SLICED dense
                         products (the projector term is then formed as exact slice products
                         and added in double-float); CS_ERR_STATE otherwise.               */,
@@ -195,7 +199,7 @@ cs_status cs_workspace_bytes(const cs_ctx* ctx, int n_s, cs_precision prec, size
  * Arlm_to_coeff), plus 1/2 Lambda X and the projector pair. X, HX: DEVICE, d x n_s,
  * leading dimension ld, element type per prec; X and HX must not overlap.
  * Requires cs_set_potential first (CS_ERR_STATE otherwise). The tensor-core kernels of
- * CS_MIXED_BF16 bound every wait; one that expires leaves HX invalid, sets the context's
+ * CS_MIXED_BF16 and of the FP64 slice products bound every wait; one that expires leaves HX invalid, sets the context's
  * device error word and still returns CS_OK (the call does not synchronise): mixed-precision
  * callers read cs_device_error after synchronising (cs_cheb_filter likewise). */
 cs_status cs_apply_H(cs_ctx* ctx, int n_s, const void* X, void* HX, long long ld,
@@ -311,7 +315,8 @@ cs_status cs_lobpcg(cs_ctx* ctx, int n_s, int n_want, double* X, long long ld, d
 cs_status cs_profile_begin(cs_ctx* ctx);
 cs_status cs_profile_end(cs_ctx* ctx, double* ms, long long* launches);
 
-/* H X like cs_apply_H, for callers that cannot allocate device memory when they call (for
+/* H X like cs_apply_H (FP64 in FP64 arithmetic at every size, so that large blocks may differ from
+ * cs_apply_H in the last bits), for callers that cannot allocate device memory when they call (for
  * example when another allocator already holds the free device memory, or when a loop must
  * not take the device-wide synchronisation of cudaMalloc/cudaFree). It needs no workspace:
  * its scratch is a 32 MiB array compiled into the library, present on every GPU that loads

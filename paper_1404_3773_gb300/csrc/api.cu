@@ -1091,9 +1091,14 @@ cs_status cs_rayleigh_ritz(cs_ctx* c, int n_s, double* X, long long ld, double* 
   int* status = reinterpret_cast<int*>((char*)work + layout(c, n_s, CS_FP64).status);
   if ((s = rr_core(c, n_s, X, ld, theta, resid, HX_out, (char*)work, st, status + 4)) != CS_OK)
     return s;
-  int hs;
-  if ((s = read_status(c, status + 4, 1, &hs, st)) != CS_OK) return s;
-  if (hs < 0) return fail(c, CS_ERR_NOT_CONVERGED, "Jacobi eigensolver did not converge");
+  // the device error word (bounded waits of the slice products) beside the eigensolver's status,
+  // in one read
+  CS_CHECK_CUDA(c, cudaMemcpyAsync(status + 5, c->dev_err, sizeof(int), cudaMemcpyDeviceToDevice,
+                                   st));
+  int hs[2];
+  if ((s = read_status(c, status + 4, 2, hs, st)) != CS_OK) return s;
+  if (hs[1] != 0) return check_dev_err(c, st);
+  if (hs[0] < 0) return fail(c, CS_ERR_NOT_CONVERGED, "Jacobi eigensolver did not converge");
   return CS_OK;
 }
 
@@ -1147,7 +1152,7 @@ cs_status cs_lanczos_bound(cs_ctx* c, int k, const double* v0, double* b, double
   *theta_min = hth[0];
   if (!std::isfinite(*b) || !std::isfinite(*theta_min))
     return fail(c, CS_ERR_NUMERIC, "Lanczos produced a non-finite bound (breakdown?)");
-  return CS_OK;
+  return check_dev_err(c, st);
 }
 
 cs_status cs_chfsi(cs_ctx* c, int n_s, int n_want, double* X, long long ld, int degree,

@@ -333,9 +333,15 @@ cs_status cs_lobpcg(cs_ctx* c, int m, int n_want, double* X, long long ld, doubl
   LB_CUDA(c, launch_copy_block<double>(S, d, X, ld, d, m, st));
   LB_CUDA(c, cudaMemcpyAsync(theta, th, m * 8, cudaMemcpyDeviceToDevice, st));
   LB_CUDA(c, cudaMemcpyAsync(resid, nrm, m * 8, cudaMemcpyDeviceToDevice, st));
+  int code = 0;  // a bounded wait of the slice products that expired
+  LB_CUDA(c, cudaMemcpyAsync(&code, c->dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   LB_CUDA(c, cudaStreamSynchronize(st));
   if (iters) *iters = it;
   if (restarts) *restarts = nrest;
+  if (code != 0) {
+    LB_CUDA(c, cudaMemsetAsync(c->dev_err, 0, sizeof(int), st));
+    return lfail(c, CS_ERR_TIMEOUT, "a bounded device wait expired (code " + std::to_string(code) + ")");
+  }
   if (result != CS_OK) return lfail(c, CS_ERR_NOT_CONVERGED, "cs_lobpcg: tolerance not reached");
   return CS_OK;
 }
