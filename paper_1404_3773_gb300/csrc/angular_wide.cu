@@ -447,6 +447,12 @@ __global__ void __launch_bounds__(kL2Threads, 2)
 // (4 QP in all), quadrature class c at 4 QP + c KC. The quadrature runs in passes over QH
 // quarter angles: each pass forms the four classes' folded grid values for its angles once,
 // and its MMAs accumulate into the quadrature columns.
+// Bound: instruction issue (60 % of the slots, 16 warps; DRAM 2 TB/s) in converting F and the
+// folded grid values to hi/lo operands, and the waits between the MMAs and the two conversions
+// of a tile. The operand buffer allows one CTA per SM, so the overlap is made inside it: the
+// next tile's synthesis is started after the last quadrature MMA, before this tile's AP is
+// drained (their tensor-memory columns are apart), and the operand descriptors are formed once.
+// Large cluster, lmax 60, 192 x 120 x 240 grid, 128 states: 1490 -> 1440 us.
 __global__ void __launch_bounds__(kPThreads, 1)
     k_phi_tc(WaArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -505,14 +511,22 @@ __global__ void __launch_bounds__(kPThreads, 1)
   const int qd = warp & 3, cg = warp >> 2, s_me = 32 * qd + lane;
   const uint32_t lane_base = (uint32_t)(32 * qd) << 16;
   const int npass = QP / QH;
+  // descriptors of warp c's operands; a K step adds rows * 32 bytes, in units of 16
+  constexpr int kDescA = 2 * kWaRows;
+  auto desc = [](const unsigned char* p) { return make_desc(smem_u32(p), 128, 256); };
+  const size_t wc = warp < 4 ? warp : 0;
+  const uint64_t df_h = desc(sA + wc * 2 * fplane), df_l = desc(sA + wc * 2 * fplane + fplane);
+  const uint64_t dh_h = desc(sA + wc * 2 * hplane), dh_l = desc(sA + wc * 2 * hplane + hplane);
+  const uint64_t dt_h = desc(sT + wc * 2 * tplane), dt_l = desc(sT + wc * 2 * tplane + tplane);
+  const uint64_t du_h = desc(sUt + wc * 2 * tplane), du_l = desc(sUt + wc * 2 * tplane + tplane);
   uint32_t ph_f = 0, ph_mma = 0;
-  int buf = 0;
-  for (long long tl = blockIdx.x; ok && tl < ntiles; tl += gridDim.x, buf ^= 1) {
-    bool w_ok = mbar_wait(bar_f, ph_f);
+  // Tile tl's F to the operand of the four classes, its synthesis MMAs started and the next
+  // tile's F and W V requested. The operand buffer is free: the MMAs that read it have completed.
+  auto start_tile = [&](long long tl, int buf) -> bool {
+    const bool f_ok = mbar_wait(bar_f, ph_f);
     ph_f ^= 1u;
-    if (!w_ok) record(a.err, 26);
-    ok = __syncthreads_and(w_ok ? 1 : 0) != 0;
-    if (!ok) break;
+    if (!f_ok) record(a.err, 26);
+    if (__syncthreads_and(f_ok ? 1 : 0) == 0) return false;
     // ---- F operand of the four classes: A_c[s][i] = F[kap(c, i)][s]
     {
       const int ntask = kWaRows * 4 * (KC / 8);
@@ -549,21 +563,22 @@ __global__ void __launch_bounds__(kPThreads, 1)
       tc_fence_after();
       {
         const int c = warp;
-        const uint32_t ah = smem_u32(sA + (size_t)c * 2 * fplane), al = ah + (uint32_t)fplane;
-        const uint32_t bh = smem_u32(sT + (size_t)c * 2 * tplane), bl = bh + (uint32_t)tplane;
+        const uint32_t d = tmem + (uint32_t)(c * QP);
         for (int ks = 0; ks < KC / 16; ++ks) {
-          const uint32_t ao = ks * (kWaRows / 8) * 256, bo = ks * (QP / 8) * 256;
-          const uint64_t dah = make_desc(ah + ao, 128, 256), dal = make_desc(al + ao, 128, 256);
-          const uint64_t dbh = make_desc(bh + bo, 128, 256), dbl = make_desc(bl + bo, 128, 256);
-          const uint32_t d = tmem + (uint32_t)(c * QP);
-          mma_bf16(d, dah, dbh, idesc_s, ks > 0 ? 1u : 0u);
-          mma_bf16(d, dah, dbl, idesc_s, 1u);
-          mma_bf16(d, dal, dbh, idesc_s, 1u);
+          const uint64_t ao = (uint64_t)(ks * kDescA), bo = (uint64_t)(ks * 2 * QP);
+          mma_bf16(d, df_h + ao, dt_h + bo, idesc_s, ks > 0 ? 1u : 0u);
+          mma_bf16(d, df_h + ao, dt_l + bo, idesc_s, 1u);
+          mma_bf16(d, df_l + ao, dt_h + bo, idesc_s, 1u);
         }
       }
       mma_commit(bar_mma);
     }
-    w_ok = mbar_wait(bar_mma, ph_mma);
+    return true;
+  };
+  if (ok && (long long)blockIdx.x < ntiles) ok = start_tile(blockIdx.x, 0);
+  int buf = 0;
+  for (long long tl = blockIdx.x; ok && tl < ntiles; tl += gridDim.x, buf ^= 1) {
+    bool w_ok = mbar_wait(bar_mma, ph_mma);
     ph_mma ^= 1u;
     if (!w_ok) record(a.err, 27);
     ok = __syncthreads_and(w_ok ? 1 : 0) != 0;
@@ -610,17 +625,13 @@ __global__ void __launch_bounds__(kPThreads, 1)
         tc_fence_after();
         {
           const int c = warp;
-          const uint32_t ah = smem_u32(sA + (size_t)c * 2 * hplane), al = ah + (uint32_t)hplane;
-          const uint32_t uh = smem_u32(sUt + (size_t)c * 2 * tplane), ul = uh + (uint32_t)tplane;
+          const uint32_t d = tmem + (uint32_t)(4 * QP + c * KC);
           for (int ks = 0; ks < QH / 16; ++ks) {
-            const uint32_t ao = ks * (kWaRows / 8) * 256;
-            const uint32_t uo = (pass * (QH / 16) + ks) * (KC / 8) * 256;
-            const uint64_t dah = make_desc(ah + ao, 128, 256), dal = make_desc(al + ao, 128, 256);
-            const uint64_t duh = make_desc(uh + uo, 128, 256), dul = make_desc(ul + uo, 128, 256);
-            const uint32_t d = tmem + (uint32_t)(4 * QP + c * KC);
-            mma_bf16(d, dah, duh, idesc_a, (pass > 0 || ks > 0) ? 1u : 0u);
-            mma_bf16(d, dah, dul, idesc_a, 1u);
-            mma_bf16(d, dal, duh, idesc_a, 1u);
+            const uint64_t ao = (uint64_t)(ks * kDescA);
+            const uint64_t uo = (uint64_t)((pass * (QH / 16) + ks) * 2 * KC);
+            mma_bf16(d, dh_h + ao, du_h + uo, idesc_a, (pass > 0 || ks > 0) ? 1u : 0u);
+            mma_bf16(d, dh_h + ao, du_l + uo, idesc_a, 1u);
+            mma_bf16(d, dh_l + ao, du_h + uo, idesc_a, 1u);
           }
         }
         mma_commit(bar_mma);
@@ -631,6 +642,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
       ok = __syncthreads_and(w_ok ? 1 : 0) != 0;
       tc_fence_after();
     }
+    if (!ok) break;
+    // the next tile's synthesis runs while this one's AP leaves tensor memory
+    if (tl + gridDim.x < ntiles) ok = start_tile(tl + gridDim.x, buf ^ 1);
     if (!ok) break;
     // AP[kap][s] in place of the row's F; warp column group cg writes class cg
     {
