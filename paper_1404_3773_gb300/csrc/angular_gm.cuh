@@ -12,12 +12,18 @@
 //                         cos/sin x even/odd-m quadrature inputs
 //   C: AP[m][p][+-][s]  = sum_q {cos|sin}(m phi_q) Wq[...][q][col], combined over j, jb
 //   D: G'[l,m][s]      += sum_p Theta_lm(t_jp) AP[m][p][parity of l+|m|][s]
-// B and C use 4 x 4 register tiles with a warp's lanes laid out 4 (rows) x 8 (columns) and
-// load the next step's operands while the current FMAs run; C groups the modes by parity
-// so one tile needs one cos and one sin input array. D accumulates the (l, m) outputs for all
-// 8 states in shared memory; an item is five l of one parity of one mode, its lanes share a
-// mode, so each AP load is a broadcast that feeds 40 FMAs, and up to lmax 31 every thread has
-// at most one item. The Legendre rows of a chunk come pre-transposed ([packed (m,l)][pair])
+// B and C are bound by the shared-memory pipe: a 16-byte load takes four wavefronts also where
+// lanes share addresses, so the bytes per FMA of a thread's tile count. Their tiles are 8 rows
+// (q or modes) x 4 columns of the cos or of the sin sums (12 operands for 32 FMAs; 4 x 4 of both
+// takes 16), with the next step's operands loaded while the current FMAs run; in B the lane
+// pair of a tile exchanges half of its sums by shuffles, in C the modes are grouped by parity so
+// a tile needs one input array. Eight consecutive lanes hold eight consecutive column blocks, so
+// a store writes 128 consecutive bytes (17.8M -> 10.0M store wavefronts against lanes that vary
+// the rows first). Per 80-state launch at lmax 30,
+// 48 radial functions: 316 us with 4 x 4 tiles, rows first; 295 columns first; 290 with the 8 x 4
+// tiles. D accumulates the (l, m) outputs for all 8 states in shared memory; an item is five l of
+// one parity of one mode, its lanes share a mode, so each AP load is a broadcast that feeds 40
+// FMAs, two states to a packed instruction, and up to lmax 31 every thread has at most one item. The Legendre rows of a chunk come pre-transposed ([packed (m,l)][pair])
 // from a table built at set-up, followed by the phi tables in their shared-memory layouts, so
 // staging either is a contiguous copy. The W V rows of a chunk are staged in the AP region
 // (free until stage C) before stage A. Both come from registers loaded during the previous
@@ -302,78 +308,86 @@ __device__ __forceinline__ void angular_gm_block(const AngArgs<float>& a, float*
     }
     __syncthreads();
     // ---- B: phi sums at the folded angles, W V, folded quadrature inputs.
-    //      Warp tile = 4 q-blocks x 8 column blocks (lanes 4 x 8).
+    //      Warp tile = 2 blocks of 8 q x {cos, sin} x 8 column blocks; the lane pair of one
+    //      block exchanges half of its sums, so each ends with the cos and sin sums of 4 q.
     {
-      const int nQB = Qp / 4, nQW = (nQB + 3) / 4;
+      const int nQB = (Qp + 7) / 8, nQW = (nQB + 1) / 2;
       constexpr int nCW = NC / 32;
+      const int odd = (lane >> 3) & 1;  // 1: the sin sums
+      const int sgn = odd ? -1 : 1;     // F(lmax + sgn m)
+      const float fs = (float)sgn;
       for (int wt = warp; wt < nQW * nCW; wt += kGmThreads / 32) {
-        const int qb = (wt % nQW) * 4 + (lane & 3);
-        const int cb = (wt / nQW) * 8 + (lane >> 2);
-        if (qb >= nQB) continue;
-        const int q0 = 4 * qb, cc = 4 * cb;
-        float Ee[4][4], Eo[4][4], Oe[4][4], Oo[4][4];
+        const int qb = min((wt % nQW) * 2 + (lane >> 4), nQB - 1);  // past the last: repeated
+        const int cb = (wt / nQW) * 8 + (lane & 7);
+        // own rows first (stored here), then the partner's; past Qp they read the next
+        // table row and are dropped
+        const int q0 = 8 * qb + 4 * odd, q1 = 8 * qb + 4 * (1 - odd), cc = 4 * cb;
+        float Xe[8][4], Xo[8][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 8; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) Ee[i][j] = Eo[i][j] = Oe[i][j] = Oo[i][j] = 0.f;
+          for (int j = 0; j < 4; ++j) Xe[i][j] = Xo[i][j] = 0.f;
         // operands of mode m are loaded while the other parity's FMAs run; rows past lmax
         // are zero padding, so the odd partner of the last even mode needs no test
-        float4 e_tc = ld4(Tb + q0), e_ts = ld4(Tb + (size_t)Lb * Qp + q0);
-        float4 e_fp = ld4(F + (size_t)lmax * NCp + cc), e_fm = e_fp;
+        const float* tb = Tb + (odd ? (size_t)Lb * Qp : 0);
+        const float* fb = F + (size_t)lmax * NCp + cc;
+        float4 e_t0 = ld4(tb + q0), e_t1 = ld4(tb + q1), e_f = ld4(fb);
         for (int m = 0; m < L; m += 2) {
           const int mo = m + 1;
-          const float4 o_tc = ld4(Tb + (size_t)mo * Qp + q0);
-          const float4 o_ts = ld4(Tb + (size_t)(Lb + mo) * Qp + q0);
-          const float4 o_fp = ld4(F + (size_t)(lmax + mo) * NCp + cc);
-          const float4 o_fm = ld4(F + (size_t)(lmax - mo) * NCp + cc);
+          const float4 o_t0 = ld4(tb + (size_t)mo * Qp + q0);
+          const float4 o_t1 = ld4(tb + (size_t)mo * Qp + q1);
+          const float4 o_f = ld4(fb + (ptrdiff_t)(sgn * mo) * NCp);
           {
-            float tc[4], ts[4], fp[4], fm[4];
-            unpack4(e_tc, tc); unpack4(e_ts, ts); unpack4(e_fp, fp); unpack4(e_fm, fm);
+            float t[8], f[4];
+            unpack4(e_t0, t); unpack4(e_t1, t + 4); unpack4(e_f, f);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                Ee[i][j] = fmaf(tc[i], fp[j], Ee[i][j]);
-                Oe[i][j] = fmaf(ts[i], fm[j], Oe[i][j]);
-              }
+              for (int j = 0; j < 4; ++j) Xe[i][j] = fmaf(t[i], f[j], Xe[i][j]);
           }
           if (m + 2 < L) {
             const int me = m + 2;
-            e_tc = ld4(Tb + (size_t)me * Qp + q0);
-            e_ts = ld4(Tb + (size_t)(Lb + me) * Qp + q0);
-            e_fp = ld4(F + (size_t)(lmax + me) * NCp + cc);
-            e_fm = ld4(F + (size_t)(lmax - me) * NCp + cc);
+            e_t0 = ld4(tb + (size_t)me * Qp + q0);
+            e_t1 = ld4(tb + (size_t)me * Qp + q1);
+            e_f = ld4(fb + (ptrdiff_t)(sgn * me) * NCp);
           }
           {
-            float tc[4], ts[4], fp[4], fm[4];
-            unpack4(o_tc, tc); unpack4(o_ts, ts); unpack4(o_fp, fp); unpack4(o_fm, fm);
+            float t[8], f[4];
+            unpack4(o_t0, t); unpack4(o_t1, t + 4); unpack4(o_f, f);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                Eo[i][j] = fmaf(tc[i], fp[j], Eo[i][j]);
-                Oo[i][j] = fmaf(ts[i], fm[j], Oo[i][j]);
-              }
+              for (int j = 0; j < 4; ++j) Xo[i][j] = fmaf(t[i], f[j], Xo[i][j]);
           }
         }
+        // the partner's sums of the own rows: Y where X holds the other of cos and sin
+        float Ye[4][4], Yo[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            Ye[i][j] = __shfl_xor_sync(0xffffffffu, Xe[4 + i][j], 8);
+            Yo[i][j] = __shfl_xor_sync(0xffffffffu, Xo[4 + i][j], 8);
+          }
+        if ((wt % nQW) * 2 + (lane >> 4) >= nQB || q0 >= Qp) continue;
         // W V of the pair's two rows at the 16 angles of the tile (staged rows; zero rows
         // stand for absent mirrors and pairs past the last)
         const int p = cb >> 2;  // 4 column blocks per pair
         const float* wr0 = AP + (size_t)(2 * p) * Np;
         const float* wr1 = wr0 + Np;
-        float wang[2][4][4];  // [row][q][angle q, N-q, h-q, h+q]
+        float wang[2][4][4];  // [row][q][angle q, N-q, h-q, h+q]; fs: see the differences below
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int q = q0 + i;
           const bool ok = q <= Q4;
           const int i0 = q, i1 = (Np - q) % Np, i2 = h - q, i3 = h + q;
           wang[0][i][0] = ok ? wr0[i0] : 0.f;
-          wang[0][i][1] = ok ? wr0[i1] : 0.f;
-          wang[0][i][2] = ok ? wr0[i2] : 0.f;
+          wang[0][i][1] = ok ? fs * wr0[i1] : 0.f;
+          wang[0][i][2] = ok ? fs * wr0[i2] : 0.f;
           wang[0][i][3] = ok ? wr0[i3] : 0.f;
           wang[1][i][0] = ok ? wr1[i0] : 0.f;
-          wang[1][i][1] = ok ? wr1[i1] : 0.f;
-          wang[1][i][2] = ok ? wr1[i2] : 0.f;
+          wang[1][i][1] = ok ? fs * wr1[i1] : 0.f;
+          wang[1][i][2] = ok ? fs * wr1[i2] : 0.f;
           wang[1][i][3] = ok ? wr1[i3] : 0.f;
         }
 #pragma unroll
@@ -384,10 +398,11 @@ __device__ __forceinline__ void angular_gm_block(const AngArgs<float>& a, float*
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const int r = j >> 1;  // columns 0,1: row j; 2,3: mirror row jb
-            const float EpE = Ee[i][j] + Eo[i][j], EmE = Ee[i][j] - Eo[i][j];
-            const float OpO = Oe[i][j] + Oo[i][j], OmO = Oe[i][j] - Oo[i][j];
-            const float g_q = wang[r][i][0] * (EpE + OpO), g_Nq = wang[r][i][1] * (EpE - OpO);
-            const float g_hm = wang[r][i][2] * (EmE - OmO), g_hp = wang[r][i][3] * (EmE + OmO);
+            // cos minus sin is fs (own minus partner's); fs is in the W V values
+            const float XpX = Xe[i][j] + Xo[i][j], XmX = Xe[i][j] - Xo[i][j];
+            const float YpY = Ye[i][j] + Yo[i][j], YmY = Ye[i][j] - Yo[i][j];
+            const float g_q = wang[r][i][0] * (XpX + YpY), g_Nq = wang[r][i][1] * (XpX - YpY);
+            const float g_hm = wang[r][i][2] * (XmX - YmY), g_hp = wang[r][i][3] * (XmX + YmY);
             const float Pp = wq * (g_q + g_Nq), Mm = wq * (g_q - g_Nq);
             const float P2 = wq * (g_hm + g_hp), M2v = wq * (g_hm - g_hp);
             c0v[j] = Pp + P2;
@@ -406,58 +421,53 @@ __device__ __forceinline__ void angular_gm_block(const AngArgs<float>& a, float*
     __syncthreads();
     // the next chunk's rows: their loads run while stages C and D compute
     if (c0 + RC < NP) fetch_chunk(c0 + RC, ch + 1);
-    // ---- C: phi quadrature of one parity class of modes per tile, combined over the mirror
-    //      rows: AP[m][p][0] = A_j + A_jb, AP[m][p][1] = A_j - A_jb. Warp tile = 4 mode
-    //      blocks x 8 column blocks.
+    // ---- C: phi quadrature of one parity class of modes, cos or sin, per tile, combined over
+    //      the mirror rows: AP[m][p][0] = A_j + A_jb, AP[m][p][1] = A_j - A_jb. Warp tile =
+    //      2 blocks of 8 modes x {cos, sin} x 8 column blocks.
     {
-      const int nMB = Lq / 4, nMW = (nMB + 3) / 4;
+      const int nE = (ne4 + 7) / 8, nMB = nE + (Lq - ne4 + 7) / 8, nMW = (nMB + 1) / 2;
       constexpr int nCW = NC / 32;
+      const int odd = (lane >> 3) & 1;  // 1: the sin sums
       for (int wt = warp; wt < nMW * nCW; wt += kGmThreads / 32) {
-        const int mb = (wt % nMW) * 4 + (lane & 3);
-        const int cb = (wt / nMW) * 8 + (lane >> 2);
+        const int mb = (wt % nMW) * 2 + (lane >> 4);
+        const int cb = (wt / nMW) * 8 + (lane & 7);
         if (mb >= nMB) continue;
-        const int mp0 = 4 * mb, cc = 4 * cb;
-        const int par = (mp0 >= ne4) ? 1 : 0;
-        const float* wc = Wq + (size_t)par * WS + cc;         // cos, parity of m
-        const float* wsn = Wq + (size_t)(2 + par) * WS + cc;  // sin, parity of m
-        float Ac[4][4], As[4][4];
+        const int par = (mb >= nE) ? 1 : 0;
+        // a block's rows past its class read other table entries and are dropped
+        const int mp0 = par ? ne4 + 8 * (mb - nE) : 8 * mb, cc = 4 * cb;
+        const int mend = par ? Lq : ne4;
+        const float* wb = Wq + (size_t)(2 * odd + par) * WS + cc;
+        const float* tb = Tc + (odd ? (size_t)(Qp + 1) * Lq : 0) + mp0;
+        float A[8][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 8; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) Ac[i][j] = As[i][j] = 0.f;
+          for (int j = 0; j < 4; ++j) A[i][j] = 0.f;
         // row Qp of Tc and Wq is zero, so the prefetch of step q + 1 needs no test
-        float4 c_tc = ld4(Tc + mp0), c_ts = ld4(Tc + (size_t)(Qp + 1) * Lq + mp0);
-        float4 c_wc = ld4(wc), c_ws = ld4(wsn);
+        const bool two = mp0 + 4 < mend;
+        const float* tb1 = tb + (two ? 4 : 0);
+        float4 c_t0 = ld4(tb), c_t1 = ld4(tb1), c_w = ld4(wb);
         for (int q = 0; q < Qp; ++q) {
-          const float4 n_tc = ld4(Tc + (size_t)(q + 1) * Lq + mp0);
-          const float4 n_ts = ld4(Tc + (size_t)(Qp + 1 + q + 1) * Lq + mp0);
-          const float4 n_wc = ld4(wc + (size_t)(q + 1) * NC);
-          const float4 n_ws = ld4(wsn + (size_t)(q + 1) * NC);
-          float tc[4], ts[4], w1[4], w2[4];
-          unpack4(c_tc, tc); unpack4(c_ts, ts); unpack4(c_wc, w1); unpack4(c_ws, w2);
+          const float4 n_t0 = ld4(tb + (size_t)(q + 1) * Lq);
+          const float4 n_t1 = ld4(tb1 + (size_t)(q + 1) * Lq);
+          const float4 n_w = ld4(wb + (size_t)(q + 1) * NC);
+          float t[8], w[4];
+          unpack4(c_t0, t); unpack4(c_t1, t + 4); unpack4(c_w, w);
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
+          for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              Ac[i][j] = fmaf(tc[i], w1[j], Ac[i][j]);
-              As[i][j] = fmaf(ts[i], w2[j], As[i][j]);
-            }
-          c_tc = n_tc; c_ts = n_ts; c_wc = n_wc; c_ws = n_ws;
+            for (int j = 0; j < 4; ++j) A[i][j] = fmaf(t[i], w[j], A[i][j]);
+          c_t0 = n_t0; c_t1 = n_t1; c_w = n_w;
         }
         const int p = cb >> 2, sp = cb & 3;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 8; ++i) {
           const int mp = mp0 + i;
           const int m = par ? 2 * (mp - ne4) + 1 : 2 * mp;
-          if (m > lmax) continue;
-          float* ac = AP + ((size_t)(lmax + m) * RC + p) * 2 * ST + 2 * sp;
-          st2(ac, Ac[i][0] + Ac[i][2], Ac[i][1] + Ac[i][3]);
-          st2(ac + ST, Ac[i][0] - Ac[i][2], Ac[i][1] - Ac[i][3]);
-          if (m > 0) {
-            float* as = AP + ((size_t)(lmax - m) * RC + p) * 2 * ST + 2 * sp;
-            st2(as, As[i][0] + As[i][2], As[i][1] + As[i][3]);
-            st2(as + ST, As[i][0] - As[i][2], As[i][1] - As[i][3]);
-          }
+          if (mp >= mend || m > lmax || (odd && m == 0)) continue;
+          float* ap = AP + ((size_t)(odd ? lmax - m : lmax + m) * RC + p) * 2 * ST + 2 * sp;
+          st2(ap, A[i][0] + A[i][2], A[i][1] + A[i][3]);
+          st2(ap + ST, A[i][0] - A[i][2], A[i][1] - A[i][3]);
         }
       }
     }
@@ -499,7 +509,12 @@ __device__ __forceinline__ void angular_gm_block(const AngArgs<float>& a, float*
 #pragma unroll
         for (int v = 0; v < kGmLq; ++v)
 #pragma unroll
-          for (int q = 0; q < ST; ++q) acc[v][q] = fmaf(pv[v][pp], av[q], acc[v][q]);
+          for (int q = 0; q < ST; q += 2) {
+            const float2 r = __ffma2_rn(make_float2(pv[v][pp], pv[v][pp]), make_float2(av[q], av[q + 1]),
+                                        make_float2(acc[v][q], acc[v][q + 1]));
+            acc[v][q] = r.x;
+            acc[v][q + 1] = r.y;
+          }
       }
 #pragma unroll
       for (int v = 0; v < kGmLq; ++v) {
