@@ -149,6 +149,9 @@ __device__ __forceinline__ df64& operator-=(df64& a, df64 b) { return a = a - b;
 // Two df64acc side by side on packed FP32 instructions (sm_100: one instruction, two lanes): the
 // same roundings per lane, half the instruction issue that bounds the double-float products.
 // Operands come as pairs of leading and trailing parts; nah = -ah, so that -p is a plain product.
+// (Host programs that use the conversions compile this header for a default architecture, which
+// lacks the packed instructions.)
+#if !defined(__CUDA_ARCH__) || __CUDA_ARCH__ >= 1000
 struct df64acc2 {
   float2 hi = {0.f, 0.f}, lo = {0.f, 0.f};
   __device__ __forceinline__ void add_prod(float2 ah, float2 nah, float2 al, float2 bh,
@@ -181,6 +184,7 @@ struct df64acc2 {
     return a.value();
   }
 };
+#endif
 
 // Multiply-add accumulator over an arithmetic type: a fused multiply-add for float and double,
 // df64acc for df64 (one renormalisation when read).
