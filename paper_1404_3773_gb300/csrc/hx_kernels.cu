@@ -1,4 +1,5 @@
-// H.X kernels for FP64 and FP32 (FMA pipes). Sec. 2.2.4 eq. matvec_final:
+// H.X kernels for FP64, double-float and FP32 on the FMA pipes (FP64 and large double-float
+// calls take sliced_hx.cu instead). Sec. 2.2.4 eq. matvec_final:
 //   H Y = 1/2 Lambda Y + forward( W V . inverse(Y) ) (+ projector pair)
 // split into three launches per block of states:
 //   k_radial_synth  : G[k][lm][s] = sum_n R_ln(r_k) X[alpha(l,m,n), s]         (eq. G_lmr)

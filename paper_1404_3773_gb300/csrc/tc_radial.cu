@@ -6,7 +6,8 @@
 // The state tile is the MMA's A operand (M = 128 columns, K = n or k), the radial table its B
 // operand (N = n_r or N rounded up to 16, at most 256), so no tile rows are wasted on the short
 // radial dimensions and, in the epilogue, a lane owns one column: the synthesis stores of G
-// coalesce across lanes, and the analysis reads and writes 16-byte runs of its column.
+// coalesce across lanes, and the analysis reads and writes 16-byte runs of its column where the
+// block is 16-byte aligned, and goes through shared memory where it is not.
 // Operands are BF16 in the canonical K-major no-swizzle layout (8-row x 16-byte core
 // matrices). Each FP32 operand is split into hi = bf16(x) and lo = bf16(x - hi); the product
 // is accumulated in FP32 tensor memory as hi*hi + hi*lo + lo*hi (split BF16), so the
