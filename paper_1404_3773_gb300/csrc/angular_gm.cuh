@@ -20,7 +20,7 @@
 // a tile needs one input array. Eight consecutive lanes hold eight consecutive column blocks, so
 // a store writes 128 consecutive bytes (17.8M -> 10.0M store wavefronts against lanes that vary
 // the rows first). Per 80-state launch at lmax 30,
-// 48 radial functions: 316 us with 4 x 4 tiles, rows first; 295 columns first; 290 with the 8 x 4
+// 48 radial functions: 316 us with 4 x 4 tiles, rows first; 295 columns first; 289 with the 8 x 4
 // tiles. D accumulates the (l, m) outputs for all 8 states in shared memory; an item is five l of
 // one parity of one mode, its lanes share a mode, so each AP load is a broadcast that feeds 40
 // FMAs, two states to a packed instruction, and up to lmax 31 every thread has at most one item. The Legendre rows of a chunk come pre-transposed ([packed (m,l)][pair])
