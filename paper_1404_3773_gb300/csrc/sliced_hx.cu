@@ -65,12 +65,29 @@ enum { OP_R1, OP_L1, OP_P1, OP_P2, OP_L2, OP_R2 };
 
 // Programmatic dependent launch (SlPlan says when): a kernel of the chain lets the next one start its prologue
 // (barriers, tensor memory, table images) at once, and touches the chain's data only when the
-// kernel before it has completed and its writes are visible.
+// kernel before it has completed and its writes are visible. A kernel that is resident early runs
+// while its predecessor still writes, so __ldg and __restrict__ are for what no kernel of a chain
+// writes (the set-up tables, W V, the weights and occupations): the read-only path needs data that
+// does not change while the kernel runs, and either lets the compiler move a load above the wait.
+// Blocks, grid functions and intermediates are read with ordinary loads through plain pointers.
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// One word of a chain's data. Volatile, so that it stays behind pdl_wait, and stated as an
+// instruction, because plain C++ loads here cost 1.0 % of an 80-state H.X at lmax 30 (1496 -> 1512
+// us) and 8 % of two states at lmax 62 (199 -> 216 us); this form takes the time of __ldg.
+__device__ __forceinline__ long long ld_chain(const long long* p) {
+  long long v;
+  asm volatile("ld.global.b64 %0, [%1];" : "=l"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_chain(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
 }
 
 // bytes of one table image: `ks` K steps, nb table rows
@@ -303,20 +320,20 @@ __device__ __forceinline__ void sl_load8(const SlArgs& a, const SlRow& w, int cl
     const double* x = a.X + (size_t)(w.l * w.l + w.mi) * a.N + (size_t)w.s * a.ld;
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      if (kb + i < a.N) v[i] = __double_as_longlong(__ldg(x + kb + i));
+      if (kb + i < a.N) v[i] = __double_as_longlong(ld_chain(x + kb + i));
   } else if constexpr (OP == OP_R2) {
     const size_t st = (size_t)a.L * a.L * a.S;
     const double* g = a.G + (size_t)(w.l * w.l + w.mi) * a.S + w.s;
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      if (kb + i < a.n_r) v[i] = __double_as_longlong(__ldg(g + (size_t)(kb + i) * st));
+      if (kb + i < a.n_r) v[i] = __double_as_longlong(ld_chain(g + (size_t)(kb + i) * st));
   } else if constexpr (OP == OP_L1) {
     const int am = w.m < 0 ? -w.m : w.m;
     const double* g = a.G + (size_t)(a.k0 + w.kp) * a.L * a.L * a.S + a.s0 + w.s;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int l = am + w.par + 2 * (kb + i);
-      if (l < a.L) v[i] = __double_as_longlong(__ldg(g + (size_t)(l * l + l + w.m) * a.S));
+      if (l < a.L) v[i] = __double_as_longlong(ld_chain(g + (size_t)(l * l + l + w.m) * a.S));
     }
   } else if constexpr (OP == OP_P1) {
     const int t = w.j < a.NP ? w.j : a.Nt - 1 - w.j;
@@ -329,7 +346,7 @@ __device__ __forceinline__ void sl_load8(const SlArgs& a, const SlRow& w, int cl
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const bool in = m0 + 2 * i <= lmax && (cls < 2 || m0 + 2 * i > 0);
-      const long long ev = in ? __ldg(e + off + i * st) : 0, ov = in ? __ldg(o + off + i * st) : 0;
+      const long long ev = in ? ld_chain(e + off + i * st) : 0, ov = in ? ld_chain(o + off + i * st) : 0;
       v[i] = ev + (ov ^ mir) - mir;
     }
   } else if constexpr (OP == OP_P2) {
@@ -337,7 +354,7 @@ __device__ __forceinline__ void sl_load8(const SlArgs& a, const SlRow& w, int cl
         a.W + (((size_t)(w.kp * a.Nt + w.j) * 4 + cls) * a.Q + kb) * a.SB + w.s;
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      if (kb + i < a.Q) v[i] = __ldg(x + i * a.SB);
+      if (kb + i < a.Q) v[i] = ld_chain(x + i * a.SB);
   } else {
     const int rs = a.M2 * a.SB;
     const long long odd = w.par ? -1 : 0;
@@ -345,8 +362,8 @@ __device__ __forceinline__ void sl_load8(const SlArgs& a, const SlRow& w, int cl
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int t = kb + i, jb = a.Nt - 1 - t;
-      const long long y = t < a.NP ? __ldg(x + t * rs) : 0;
-      const long long z = t < a.NP && jb != t ? __ldg(x + jb * rs) : 0;
+      const long long y = t < a.NP ? ld_chain(x + t * rs) : 0;
+      const long long z = t < a.NP && jb != t ? ld_chain(x + jb * rs) : 0;
       v[i] = y + (z ^ odd) - odd;
     }
   }
@@ -427,9 +444,9 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
     int rowsc = 0;  // F64: exponent E of the row; else: shift to 54 bits
     // ---- scale of the row
     if constexpr (OP == OP_L1) {
-      if (w.live) rowsc = __ldg(a.EG + (size_t)(a.k0 + w.kp) * a.S + a.s0 + w.s);
+      if (w.live) rowsc = a.EG[(size_t)(a.k0 + w.kp) * a.S + a.s0 + w.s];
     } else if constexpr (OP == OP_P2) {
-      if (w.live) rowsc = __ldg(a.shP + (size_t)(w.kp * a.Nt + w.j) * a.SB + w.s);
+      if (w.live) rowsc = a.shP[(size_t)(w.kp * a.Nt + w.j) * a.SB + w.s];
     } else {
       int mx = -kBig;
       if constexpr (OP == OP_P1) {
@@ -442,7 +459,7 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
           const long long mir = w.j >= a.NP ? -1 : 0;
 #pragma unroll 8
           for (int kap = half; kap < a.M2; kap += 2, e += st) {
-            const long long ev = __ldg(e), ov = __ldg(e + od);
+            const long long ev = ld_chain(e), ov = ld_chain(e + od);
             const long long v = ev + (ov ^ mir) - mir;
             acc |= (unsigned long long)(v ^ (v >> 63));
           }
@@ -490,12 +507,12 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
       nhi = w.live ? (a.L - m0 + 1) / 2 : 0;
       // results in the unit of the node's largest row (rows of zeros: no shift)
       if (w.live)
-        ush = max(0, min(63, __ldg(a.U + w.kp * a.SB + w.s) -
-                                 __ldg(a.uP + (size_t)(w.kp * a.Nt + w.j) * a.SB + w.s)));
+        ush = max(0, min(63, a.U[w.kp * a.SB + w.s] -
+                                 a.uP[(size_t)(w.kp * a.Nt + w.j) * a.SB + w.s]));
     } else if constexpr (OP == OP_L2) {
       // unit of G', which is left scaled by the radial table's power of two of its node
       if (w.live)
-        ush = __ldg(a.U + w.kp * a.SB + w.s) - rowsc + kFix - 56 - __ldg(a.rexp + a.k0 + w.kp);
+        ush = a.U[w.kp * a.SB + w.s] - rowsc + kFix - 56 - __ldg(a.rexp + a.k0 + w.kp);
     } else if constexpr (OP == OP_P1) {
       out = a.W + (size_t)(w.kp * a.Nt + w.j) * 4 * a.Q * a.SB + w.s;
       ost = a.SB;
@@ -674,7 +691,7 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
       // unit of the row's class sums: the operand's unit 2^(E_G + F1 - 56 - shift), less 2 bits
       if (w.live && half == 0)
         a.eW[(size_t)(w.kp * a.Nt + w.j) * a.SB + w.s] =
-            __ldg(a.EG + (size_t)(a.k0 + w.kp) * a.S + a.s0 + w.s) + a.F1 - 56 - rowsc +
+            a.EG[(size_t)(a.k0 + w.kp) * a.S + a.s0 + w.s] + a.F1 - 56 - rowsc +
             kFix - 56;
     }
   }
@@ -703,13 +720,11 @@ __device__ __forceinline__ long long mul_hi(long long f, long long w) {
 // sums, times W V (integer of 62 bits below the row's power of two), folded back into the four
 // classes in place; then the row's shift to 54 bits, its unit after P2 and the node's largest.
 // A CTA holds 32 (row, state) pairs; its 8 warps take the quarter angles q = warp, warp + 8, ...
-__global__ void __launch_bounds__(256) k_sl_pointwise(long long* __restrict__ W, const int* eW,
+__global__ void __launch_bounds__(256) k_sl_pointwise(long long* W, const int* eW,
                                                       const long long* __restrict__ wv,
                                                       const int* __restrict__ ewv, int rows,
                                                       int SB, int Nt, int Np, int Q, int k0,
-                                                      int* __restrict__ shP,
-                                                      int* __restrict__ uP,
-                                                      int* __restrict__ U) {
+                                                      int* shP, int* uP, int* U) {
   pdl_trigger();
   pdl_wait();
   __shared__ int red[8][32];
@@ -764,12 +779,10 @@ __global__ void __launch_bounds__(256) k_sl_pointwise(long long* __restrict__ W,
 
 // The folded classes of grid functions g[s][k][j][q] times the row's quadrature weight, as the
 // pointwise pass leaves them: one warp per (grid row, state), lanes over the quarter angles.
-__global__ void __launch_bounds__(256) k_sl_fold(const double* __restrict__ g,
+__global__ void __launch_bounds__(256) k_sl_fold(const double* g,
                                                  const double* __restrict__ wkj, int rows, int SB,
                                                  int s0, int k0, int Nt, int Np, int Q, int n_r,
-                                                 long long* __restrict__ W,
-                                                 int* __restrict__ shP, int* __restrict__ uP,
-                                                 int* __restrict__ U) {
+                                                 long long* W, int* shP, int* uP, int* U) {
   pdl_trigger();
   pdl_wait();
   const int lane = threadIdx.x & 31;
@@ -788,7 +801,7 @@ __global__ void __launch_bounds__(256) k_sl_fold(const double* __restrict__ g,
     const int at[4] = {q, q == 0 ? 0 : Np - q, h - q, h + q};
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      v[u][c] = q < Q ? __ldg(x + at[c]) * wt : 0.0;
+      v[u][c] = q < Q ? ld_chain(x + at[c]) * wt : 0.0;
       mx = max(mx, (int)((__double_as_longlong(v[u][c]) >> 52) & 0x7FF));
     }
   }
@@ -826,10 +839,9 @@ __global__ void __launch_bounds__(256) k_sl_fold(const double* __restrict__ g,
 
 // Grid values f[s][k][j][q] from the class sums: one warp per (grid row, state), the CTA's warps
 // on consecutive states so that they share the sectors of W.
-__global__ void __launch_bounds__(256) k_sl_grid(const long long* __restrict__ W,
-                                                 const int* __restrict__ eW, int rows, int SB,
-                                                 int s0, int k0, int Nt, int Np, int Q, int n_r,
-                                                 double* __restrict__ f) {
+__global__ void __launch_bounds__(256) k_sl_grid(const long long* W, const int* eW, int rows,
+                                                 int SB, int s0, int k0, int Nt, int Np, int Q,
+                                                 int n_r, double* f) {
   pdl_trigger();
   pdl_wait();
   const int lane = threadIdx.x & 31;
@@ -842,8 +854,7 @@ __global__ void __launch_bounds__(256) k_sl_grid(const long long* __restrict__ W
   const int h = Np / 2, u = eW[i];
   for (int q = lane; q < Q; q += 32) {
     const long long* p = x + (size_t)q * SB;
-    const long long c0 = __ldg(p), c1 = __ldg(p + cs), c2 = __ldg(p + 2 * cs),
-                    c3 = __ldg(p + 3 * cs);
+    const long long c0 = ld_chain(p), c1 = ld_chain(p + cs), c2 = ld_chain(p + 2 * cs), c3 = ld_chain(p + 3 * cs);
     const long long ep = c0 + c1, em = c0 - c1, op = c2 + c3, om = c2 - c3;
     y[q] = to_f64(ep + op, u);
     if (q > 0) y[Np - q] = to_f64(ep - op, u);
@@ -858,11 +869,10 @@ __global__ void __launch_bounds__(256) k_sl_grid(const long long* __restrict__ W
 // the four mirror angles of every quarter angle for 32 states at a time (lanes over the states),
 // through shared memory to one thread per angle. A state's power of two goes into its weight, so
 // that the squares need three FP64 operations per value; the FP64 pipe is what bounds this pass.
-__global__ void __launch_bounds__(256) k_sl_density(const long long* __restrict__ W,
-                                                    const int* __restrict__ eW, int SB, int Nt,
-                                                    int Np, int Q, int k0,
-                                                    const double* __restrict__ occ,
-                                                    double* __restrict__ rho, int accumulate) {
+__global__ void __launch_bounds__(256) k_sl_density(const long long* W, const int* eW, int SB,
+                                                    int Nt, int Np, int Q, int k0,
+                                                    const double* __restrict__ occ, double* rho,
+                                                    int accumulate) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ double dsm[];  // [4 Q][33], then weights [32]
@@ -886,10 +896,10 @@ __global__ void __launch_bounds__(256) k_sl_density(const long long* __restrict_
       long long c0 = 0, c1 = 0, c2 = 0, c3 = 0;
       if (live) {
         const long long* p = x + (size_t)q * SB + s;
-        c0 = __ldg(p);
-        c1 = __ldg(p + cs);
-        c2 = __ldg(p + 2 * cs);
-        c3 = __ldg(p + 3 * cs);
+        c0 = ld_chain(p);
+        c1 = ld_chain(p + cs);
+        c2 = ld_chain(p + 2 * cs);
+        c3 = ld_chain(p + 3 * cs);
       }
       const long long ep = c0 + c1, em = c0 - c1, op = c2 + c3, om = c2 - c3;
       const long long f[4] = {ep + op, ep - op, em - om, em + om};
@@ -919,8 +929,7 @@ __global__ void __launch_bounds__(256) k_sl_density(const long long* __restrict_
 }
 
 // E_G[k][s]: 2^E above every |G[k][lm][s]|
-__global__ void __launch_bounds__(256) k_sl_gexp(const double* __restrict__ G, int L2, int S,
-                                                 int* __restrict__ EG) {
+__global__ void __launch_bounds__(256) k_sl_gexp(const double* G, int L2, int S, int* EG) {
   pdl_trigger();
   pdl_wait();
   __shared__ int red[8][32];
@@ -929,7 +938,7 @@ __global__ void __launch_bounds__(256) k_sl_gexp(const double* __restrict__ G, i
   if (s < S) {
     const double* g = G + (size_t)k * L2 * S + s;
     for (int lm = wp; lm < L2; lm += 8)
-      mx = max(mx, (int)((__double_as_longlong(__ldg(g + (size_t)lm * S)) >> 52) & 0x7FF));
+      mx = max(mx, (int)((__double_as_longlong(ld_chain(g + (size_t)lm * S)) >> 52) & 0x7FF));
   }
   red[wp][threadIdx.x & 31] = mx;
   __syncthreads();
