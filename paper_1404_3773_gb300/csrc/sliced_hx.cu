@@ -42,6 +42,7 @@
 
 #include "cs_internal.h"
 #include "hx_kernels.cuh"
+#include "image_ring.cuh"
 #include "ozaki_split.cuh"
 #include "sliced_hx.h"
 #include "tc_common.cuh"
@@ -417,21 +418,20 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
   // table images: [table][column block][K chunk]
   const size_t img_full = (size_t)2 * kBStep;
   const size_t tab_block = img_full * (nch - 1) + (size_t)lastks * kBStep;
-  int slot = 0;                 // slot and parity of the current step's image
-  uint32_t ph_b = 0, ph_mma = 0;
-  int pending = 0;              // images issued and not yet waited for (thread 0)
-  auto issue_b = [&](int table, int st, int ch, int sl) {
+  int step = 0, issued = 0;     // steps begun; images requested (thread 0); see image_ring.cuh
+  auto issue_b = [&](int table, int st, int ch) {
+    const int sl = image_slot(issued);
     const uint32_t bytes = (uint32_t)(ks_of(ch) * kBStep);
     const uint32_t b = smem_u32(&bar_b[sl]);
     mbar_expect_tx(b, bytes);
     bulk_g2s(sB + (uint32_t)sl * bslot,
              a.tab + ((size_t)table * nsteps + st) * tab_block + (size_t)ch * img_full, bytes, b);
-    ++pending;
+    ++issued;
   };
   SlRow w;
   int table;
   sl_locate<OP>(a, t0, r, w, table);
-  if (tid == 0 && t0 < t1) issue_b(table, 0, 0, 0);
+  if (tid == 0 && t0 < t1) issue_b(table, 0, 0);
   pdl_wait();
   if constexpr (OP == OP_L1)  // the units' maxima of the chunk start from nothing
     for (int i = blockIdx.x * kSlThreads + tid; i < a.kc * a.SB; i += gridDim.x * kSlThreads)
@@ -565,22 +565,21 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
         if (tid == 0) {
           // the next step's image: the MMAs that read that slot have completed
           if (ch + 1 < nch) {
-            issue_b(table, st, ch + 1, slot ^ 1);
+            issue_b(table, st, ch + 1);
           } else if (st + 1 < nsteps) {
-            issue_b(table, st + 1, 0, slot ^ 1);
+            issue_b(table, st + 1, 0);
           } else if (tile + 1 < t1) {
             SlRow wn;
             int tn;
             sl_locate<OP>(a, tile + 1, 0, wn, tn);
-            issue_b(tn, 0, 0, slot ^ 1);
+            issue_b(tn, 0, 0);
           }
           tc_fence_after();
-          if (!mbar_wait(smem_u32(&bar_b[slot]), ph_b)) {
+          if (!mbar_wait(smem_u32(&bar_b[image_slot(step)]), image_parity(step))) {
             atomicCAS(a.err, 0, 41);
             good = false;
           } else {
-            --pending;
-            const uint32_t b0 = sB + (uint32_t)slot * bslot;
+            const uint32_t b0 = sB + (uint32_t)image_slot(step) * bslot;
             for (int s = 0; s < ks; ++s) {
               const uint32_t ab = sA + s * kDig * kADigit, bb = b0 + s * kBStep;
               auto mma = [&](int i, int j, int cnt, uint32_t accum) {
@@ -600,13 +599,11 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
           }
           mma_commit(smem_u32(&bar_mma));
         }
-        ph_b ^= (uint32_t)slot;  // a slot's parity changes every second step
-        slot ^= 1;
-        if (!mbar_wait(smem_u32(&bar_mma), ph_mma)) {
+        if (!mbar_wait(smem_u32(&bar_mma), mma_parity(step))) {
           atomicCAS(a.err, 0, 42);
           good = false;
         }
-        ph_mma ^= 1u;
+        ++step;
         tc_fence_after();
         if (!drain) continue;
         // ---- drain: 4 columns at a time
@@ -695,12 +692,12 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
             kFix - 56;
     }
   }
-  // after an expired wait, table images still on their way land before the CTA exits
-  if (!ok && tid == 0)
-    for (int i = 0; i < 2; ++i) {
-      const int sl = slot ^ i;
-      if (pending > i) mbar_wait(smem_u32(&bar_b[sl]), i ? ph_b ^ (uint32_t)sl : ph_b);
-    }
+  // after an expired wait: what is still on its way into this CTA's memory lands before the exit
+  if (tid == 0 && (!good || issued != step))
+    settle_images(
+        step, issued,
+        [&](int sl, uint32_t parity) { mbar_wait(smem_u32(&bar_b[sl]), parity); },
+        [&](uint32_t parity) { mbar_wait(smem_u32(&bar_mma), parity); });
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, kCols);

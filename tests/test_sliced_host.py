@@ -1,6 +1,10 @@
 """Host checks of the slice-product kernels (csrc/sliced_hx.cu)."""
 import os
 import re
+import shutil
+import subprocess
+
+import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SRC = os.path.join(ROOT, "paper_1404_3773_gb300", "csrc", "sliced_hx.cu")
@@ -32,3 +36,22 @@ def test_chain_data_is_read_with_ordinary_loads():
         for name in re.findall(r"__restrict__\s+(\w+)", params):
             assert name in CONSTANT, f"__restrict__ {name}"
     assert early == 6  # k_sl, pointwise, fold, grid, density, gexp
+
+
+def test_images_and_mmas_settle_after_an_expired_wait(tmp_path):
+    """Whichever wait of whichever step expires, a CTA leaves with no bulk copy into its shared
+    memory and no MMA on its tensor memory still open. A host program on modelled barriers."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not found")
+    # the kernel takes its slots, parities and last waits from the checked header
+    code = _code()
+    for use in ("image_slot(issued)", "image_slot(step)", "image_parity(step)", "mma_parity(step)",
+                "settle_images("):
+        assert use in code, use
+    src = os.path.join(os.path.dirname(__file__), "native", "image_ring_check.cu")
+    exe = str(tmp_path / "image_ring_check")
+    subprocess.run([nvcc, "-O2", "-std=c++17", "-o", exe, src], check=True, capture_output=True,
+                   timeout=300)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout[-2000:]
