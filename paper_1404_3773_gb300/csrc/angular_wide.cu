@@ -34,6 +34,7 @@
 
 #include "cs_internal.h"
 #include "hx_kernels.cuh"
+#include "image_ring.cuh"
 #include "tc_common.cuh"
 
 namespace cs {
@@ -526,7 +527,10 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const bool f_ok = mbar_wait(bar_f, ph_f);
     ph_f ^= 1u;
     if (!f_ok) record(a.err, 26);
-    if (__syncthreads_and(f_ok ? 1 : 0) == 0) return false;
+    if (__syncthreads_and(f_ok ? 1 : 0) == 0) {
+      ph_f = given_up(ph_f);
+      return false;
+    }
     // ---- F operand of the four classes: A_c[s][i] = F[kap(c, i)][s]
     {
       const int ntask = kWaRows * 4 * (KC / 8);
@@ -665,8 +669,16 @@ __global__ void __launch_bounds__(kPThreads, 1)
     }
     tc_fence_before();
   }
-  // a bulk copy issued for a tile this CTA did not reach (error exit) must land before exit
-  if (!ok && tid == 0) mbar_wait(bar_f, ph_f);
+  // Error exit: nothing may still be on its way into this CTA's memory when it leaves. Waits once
+  // more, bounded, for the tables, the last MMAs and F, where the parities name what was given up
+  // or is one tile ahead; completed phases return at once. (After MMAs given up in a last tile no F
+  // is ahead and that wait runs to its limit: keeping track of it in the loop costs 0.4 to 1.7 % of
+  // the H.X, by the registers it takes.)
+  if (!ok && tid == 0) {
+    mbar_wait(bar_tab, 0);
+    mbar_wait(bar_mma, given_up(ph_mma));
+    mbar_wait(bar_f, ph_f);
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, tcols);

@@ -1,4 +1,5 @@
-// Table images streamed through two shared-memory slots by bulk copies (sliced_hx.cu; internal).
+// What a CTA still has in flight when it leaves after an expired wait (internal).
+// Table images streamed through two shared-memory slots by bulk copies (sliced_hx.cu):
 // Step i of a CTA uses image i: slot i & 1, phase i >> 1 of that slot's mbarrier; its MMAs complete
 // phase i of the MMA barrier. A wait on a parity whose phase is not the next one returns at once,
 // so whoever waits for a copy has to name the step it belongs to.
@@ -13,6 +14,10 @@ __host__ __device__ constexpr uint32_t image_parity(int step) {
   return (uint32_t)(step >> 1) & 1u;
 }
 __host__ __device__ constexpr uint32_t mma_parity(int step) { return (uint32_t)step & 1u; }
+
+// One barrier whose phases are requested and waited for in turn, the parity moving on after each
+// wait: the phase that a wait has just given up.
+__host__ __device__ constexpr uint32_t given_up(uint32_t next_parity) { return next_parity ^ 1u; }
 
 // Before a CTA frees its tensor memory and exits after `step` steps and `issued` images: waits for
 // the last step's MMAs and image, whose own waits may have expired, and for the images requested

@@ -49,6 +49,11 @@ def test_images_and_mmas_settle_after_an_expired_wait(tmp_path):
     for use in ("image_slot(issued)", "image_slot(step)", "image_parity(step)", "mma_parity(step)",
                 "settle_images("):
         assert use in code, use
+    with open(os.path.join(os.path.dirname(SRC), "angular_wide.cu")) as f:
+        phi = f.read().split("k_phi_tc(WaArgs a) {")[1].split("\nvoid residency")[0]
+    for use in ("mbar_wait(bar_mma, given_up(ph_mma));\n    mbar_wait(bar_f, ph_f);",
+                "ph_f = given_up(ph_f);\n      return false;", "mbar_wait(bar_tab, 0);\n"):
+        assert use in phi, use
     src = os.path.join(os.path.dirname(__file__), "native", "image_ring_check.cu")
     exe = str(tmp_path / "image_ring_check")
     subprocess.run([nvcc, "-O2", "-std=c++17", "-o", exe, src], check=True, capture_output=True,
