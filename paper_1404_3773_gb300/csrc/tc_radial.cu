@@ -7,7 +7,7 @@
 // operand (N = n_r or N rounded up to 16, at most 256), so no tile rows are wasted on the short
 // radial dimensions and, in the epilogue, a lane owns one column: the synthesis stores of G
 // coalesce across lanes, and the analysis reads and writes 16-byte runs of its column where the
-// block is 16-byte aligned, and goes through shared memory where it is not.
+// block is 16-byte aligned, and mostly goes through shared memory where it is not.
 // Operands are BF16 in the canonical K-major no-swizzle layout (8-row x 16-byte core
 // matrices). Each FP32 operand is split into hi = bf16(x) and lo = bf16(x - hi); the product
 // is accumulated in FP32 tensor memory as hi*hi + hi*lo + lo*hi (split BF16), so the
@@ -95,6 +95,16 @@ __global__ void __launch_bounds__(kThreads) k_tc_radial(TcShape sh,
                         reinterpret_cast<uintptr_t>(ep.half_lambda) |
                         reinterpret_cast<uintptr_t>(ep.kb) | reinterpret_cast<uintptr_t>(ep.src) |
                         reinterpret_cast<uintptr_t>(ep.Yprev)) & 15) == 0;
+  // Without that alignment the tile passes through shared memory (below), which wins by what it
+  // saves in single-word accesses: with the recurrence term always, from about 5 functions per l
+  // on (16 states, lmax 8 .. 30: 11.7 / 12.9 us at N = 6, 24.3 / 34.3 at 42, 48.6 / 92.8 at 125).
+  // Without that term, where no SM has more than one tile, the pass only adds latency: direct 12.0
+  // us against 14.0 at lmax 6, N = 17, 80 states, 16.1 / 18.1 at lmax 12, N = 33, 75.5 / 81.5 at
+  // N = 250; from two tiles per SM on it wins there too (31.6 / 27.6 at 372 tiles), and with one or
+  // two states, whose tiles have few live columns, at any count (38.6 / 22.2 at N = 125).
+  const bool recur = ep.mode == EP_CHEB && ep.Yprev;
+  const bool direct = MODE == 1 && !vec_ep &&
+                      (recur ? sh.N <= 4 : gridDim.x <= 152 && (sh.S > 2 || sh.N <= 8));
   const uint32_t bar_tma = smem_u32(&bars[0]);
   const uint32_t bar_mma = smem_u32(&bars[1]);
   const uint32_t tcols = tmem_cols_for(rows);
@@ -245,7 +255,7 @@ __global__ void __launch_bounds__(kThreads) k_tc_radial(TcShape sh,
       }
     }
   }
-  if (MODE == 1 && ok && vec_ep) {
+  if (MODE == 1 && ok && (vec_ep || direct)) {
     // weight of the residual-form source term of this column (0 when there is none)
     const float sw = (ep.src && c < ncol) ? ep.src_w[s] : 0.f;
     for (int rb = 0; rb < rows; rb += 16) {
@@ -254,7 +264,7 @@ __global__ void __launch_bounds__(kThreads) k_tc_radial(TcShape sh,
       if (c >= ncol) continue;
       // Z[alpha(l, mi, n), s] for n = rb .. rb + 15 (contiguous in n)
       const size_t a0 = (size_t)(l * l + mi) * sh.N;
-      if (rb + 16 <= Mout) {
+      if (vec_ep && rb + 16 <= Mout) {
         // 16-byte runs: four float4 of each operand (a0 + rb, s ld, s ld_out multiples of 4)
         const size_t a = a0 + rb;
         const size_t o = a + (size_t)s * ep.ld_out;
@@ -334,7 +344,7 @@ __global__ void __launch_bounds__(kThreads) k_tc_radial(TcShape sh,
       }
     }
   }
-  if (MODE == 1 && ok && !vec_ep) {
+  if (MODE == 1 && ok && !vec_ep && !direct) {
     // Z[alpha(l, mi, n), s] is contiguous in n, a thread's column is not contiguous with its
     // neighbours': the tile goes through shared memory (the operand buffers, now free) so that
     // the block, the recurrence term and the output are read and written along n, whatever their
