@@ -145,7 +145,7 @@ cs_status cs_set_projectors(cs_ctx* ctx, int n_p, const double* p_coef, const do
 /* Forward basis transform (Sec. 2.2.2 eqs. Ar_lm, Arlm_to_coeff) of n grid functions:
  * g: DEVICE [n][N_r][N_theta][N_phi] doubles; coef: DEVICE d x n column-major with
  * leading dimension ld >= d; coef = B^T diag(W) g. work: DEVICE, at least
- * cs_workspace_bytes(ctx, n, CS_FP64) bytes. */
+ * cs_workspace_bytes(ctx, n, CS_FP64) bytes. Expired device waits: as cs_apply_H. */
 cs_status cs_forward_transform(cs_ctx* ctx, int n, const double* g, double* coef, long long ld,
                                void* work, cs_stream stream);
 
@@ -199,9 +199,11 @@ cs_status cs_workspace_bytes(const cs_ctx* ctx, int n_s, cs_precision prec, size
  * Arlm_to_coeff), plus 1/2 Lambda X and the projector pair. X, HX: DEVICE, d x n_s,
  * leading dimension ld, element type per prec; X and HX must not overlap.
  * Requires cs_set_potential first (CS_ERR_STATE otherwise). The tensor-core kernels of
- * CS_MIXED_BF16 and of the FP64 slice products bound every wait; one that expires leaves HX invalid, sets the context's
- * device error word and still returns CS_OK (the call does not synchronise): mixed-precision
- * callers read cs_device_error after synchronising (cs_cheb_filter likewise). */
+ * CS_MIXED_BF16 and of the slice products (CS_FP64, CS_DF64) bound every wait; one that expires
+ * leaves HX invalid, sets the context's device error word and still returns CS_OK (the call does
+ * not synchronise): callers read cs_device_error after synchronising, or meet CS_ERR_TIMEOUT in
+ * the next call that reads the word. cs_cheb_filter, cs_cheb_filter_ritz and the transforms
+ * likewise. */
 cs_status cs_apply_H(cs_ctx* ctx, int n_s, const void* X, void* HX, long long ld,
                      cs_precision prec, void* work, cs_stream stream);
 
@@ -380,8 +382,9 @@ cs_status cs_batch_set_precision(cs_batch* batch, cs_precision prec);
 const char* cs_batch_last_error(const cs_batch* batch);
 
 /* Device error word of the context (synchronising): 0 if no kernel reported a problem, else
- * the code of the first bounded wait that expired (tensor-core path). Reading clears it. A
- * non-zero word is also reported as CS_ERR_TIMEOUT by the next synchronising call. */
+ * the code of the first bounded wait that expired (tensor-core kernels). Reading clears it. A
+ * non-zero word is also reported as CS_ERR_TIMEOUT by the next call among cs_rayleigh_ritz,
+ * cs_lanczos_bound, cs_chfsi and its steps, cs_lobpcg, cs_grid_integrals and cs_scf_step. */
 cs_status cs_device_error(cs_ctx* ctx, int* code);
 
 /* Last error message of the context (static storage inside ctx; "" if none). A NULL ctx

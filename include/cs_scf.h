@@ -41,7 +41,11 @@ cs_status cs_scf_workspace_bytes(const cs_ctx* ctx, size_t* bytes);
  * column s (eq. density_expression, spin-unpolarised; Sec. 2.2.5 transform method).
  * X: DEVICE FP64 d x n_s, leading dimension ld >= d. occ: DEVICE n_s doubles (0..1).
  * rho: DEVICE N_g doubles (written; no accumulation across calls). States are processed in
- * chunks, and the sum over s runs in state order (deterministic). */
+ * chunks, and the sum over s runs in state order (deterministic).
+ * Blocks that take CS_FP64's slice products run kernels with bounded waits (as cs_hartree does):
+ * one that expires leaves rho invalid, sets the context's device error word and still returns
+ * CS_OK, because the call does not synchronise. cs_device_error tells, and cs_grid_integrals
+ * (and with it cs_scf_step) reports it as CS_ERR_TIMEOUT. */
 cs_status cs_density(cs_ctx* ctx, int n_s, const double* X, long long ld, const double* occ,
                      double* rho, void* work, cs_stream stream);
 
@@ -53,7 +57,7 @@ cs_status cs_density(cs_ctx* ctx, int n_s, const double* X, long long ld, const 
  * which equals the Laplace-expansion integral of eq. zeta_definition exactly. The first term
  * is the Dirichlet eigenfunction solution; the second is the harmonic term that carries the
  * multipole moment to the boundary.
- * rho, vh: DEVICE N_g doubles; they must not overlap. */
+ * rho, vh: DEVICE N_g doubles; they must not overlap. Expired waits: as cs_density. */
 cs_status cs_hartree(cs_ctx* ctx, const double* rho, double* vh, void* work, cs_stream stream);
 
 /* Spin-unpolarised LDA at every grid point.
@@ -67,7 +71,9 @@ cs_status cs_lda_xc(cs_ctx* ctx, const double* rho, double* exc, double* vxc,
 /* out[i] = sum_g W_g f[i][g] g[i][g] for i < n <= CS_GRID_INTEGRALS_MAX, with the grid
  * quadrature weights W (w_r w_theta 2 pi / N_phi).
  * f, g: HOST arrays of n DEVICE pointers to N_g doubles; a NULL g[i] means 1.
- * out: HOST n doubles. The reduction order is fixed (deterministic). Synchronising. */
+ * out: HOST n doubles. The reduction order is fixed (deterministic). Synchronising; a device
+ * error word left by an earlier call (cs_density, cs_hartree, ...) is read and cleared, and the
+ * call then returns CS_ERR_TIMEOUT and leaves out as it was. */
 cs_status cs_grid_integrals(cs_ctx* ctx, int n, const double* const* f,
                             const double* const* g, double* out, void* work, cs_stream stream);
 
@@ -155,7 +161,8 @@ cs_status cs_scf_work_bytes(const cs_scf* s, size_t* bytes);
  * 5. Anderson-mix v_in with v_out = v_ext + V_H + v_xc.
  * X receives the Ritz vectors. theta, resid: DEVICE n_s doubles. rep: HOST, filled.
  * Synchronising. CS_ERR_NOT_CONVERGED is not returned; max_resid reports the eigensolver's
- * state. */
+ * state. CS_ERR_TIMEOUT (an expired device wait, in the density or the Hartree potential too)
+ * leaves v_in, the mixer and the iteration count as they were: the step can be repeated. */
 cs_status cs_scf_step(cs_scf* s, double* X, long long ld, double* theta, double* resid,
                       void* work, cs_stream stream, cs_scf_report* rep);
 /* Copies one of the SCF state's grid functions into out (DEVICE, N_g doubles), enqueued on

@@ -80,7 +80,8 @@ ScfLayout scf_layout(const cs_ctx* c) {
   o.coef = take((size_t)H.d * 8);
   o.alm = take(L2 * 8);
   o.G1 = take((size_t)H.n_r * L2 * 8);
-  o.partial = take((size_t)(kDotBlocks + 1) * CS_GRID_INTEGRALS_MAX * 8);  // partials, results
+  // partials, results, device error word
+  o.partial = take(((size_t)(kDotBlocks + 1) * CS_GRID_INTEGRALS_MAX + 1) * 8);
   o.slG = take(c->sliced_ok ? (size_t)H.n_r * L2 * kSlChunk * 8 : 0);
   o.slw = take(c->sliced_ok ? sliced_hx_work_bytes(H.L, H.n_r, H.n_theta, H.n_phi, kSlChunk) : 0);
   o.total = off;
@@ -214,9 +215,11 @@ __global__ void __launch_bounds__(kDotThreads) k_dot_partial(DotArgs a, const do
   }
 }
 
-__global__ void k_dot_reduce(const double* __restrict__ partial, int n, int nb,
+// and the device error word beside the results, so that one copy brings both
+__global__ void k_dot_reduce(const double* __restrict__ partial, int n, int nb, const int* err,
                              double* __restrict__ out) {
   const int i = threadIdx.x;
+  if (i == CS_GRID_INTEGRALS_MAX) out[i] = (double)*err;
   if (i >= n) return;
   double s = 0.0;
   for (int b = 0; b < nb; ++b) s += partial[(size_t)i * nb + b];
@@ -482,11 +485,20 @@ cs_status cs_grid_integrals(cs_ctx* c, int n, const double* const* f, const doub
   k_dot_partial<<<kDotBlocks, kDotThreads, 0, st>>>(a, c->d64.wkj, c->host.n_phi, n_grid(c),
                                                     partial);
   SCF_CUDA(c, cudaGetLastError());
-  k_dot_reduce<<<1, 32, 0, st>>>(partial, n, kDotBlocks, res);
+  k_dot_reduce<<<1, 32, 0, st>>>(partial, n, kDotBlocks, c->dev_err, res);
   SCF_CUDA(c, cudaGetLastError());
   c->launches += 2;
-  SCF_CUDA(c, cudaMemcpyAsync(out, res, n * sizeof(double), cudaMemcpyDeviceToHost, st));
+  double h[CS_GRID_INTEGRALS_MAX + 1];
+  SCF_CUDA(c, cudaMemcpyAsync(h, res, sizeof(h), cudaMemcpyDeviceToHost, st));
   SCF_CUDA(c, cudaStreamSynchronize(st));
+  // the grid functions may come from kernels whose bounded waits expired (density, Hartree)
+  const int code = (int)h[CS_GRID_INTEGRALS_MAX];
+  if (code != 0) {
+    SCF_CUDA(c, cudaMemsetAsync(c->dev_err, 0, sizeof(int), st));
+    return sfail(c, CS_ERR_TIMEOUT,
+                 "a bounded device wait expired (code " + std::to_string(code) + ")");
+  }
+  std::copy(h, h + n, out);
   return CS_OK;
 }
 
@@ -667,6 +679,7 @@ struct cs_scf {
   double* v0 = nullptr;
   cs_mixer* mixer = nullptr;
   int iteration = 0;
+  bool have_v_in = false;  // v_in holds a valid potential (rho may no longer be the first density)
   double e_prev = 0.0;
   std::vector<double> theta_h, occ_h, resid_h;
 };
@@ -739,7 +752,7 @@ cs_status cs_scf_step(cs_scf* S, double* X, long long ld, double* theta, double*
   const cs_scf_params& p = S->p;
   cudaStream_t st = (cudaStream_t)stream;
   const long long ng = S->ng;
-  if (S->iteration == 0) {  // v_in = v_ext + V_H[rho0] + v_xc[rho0]
+  if (!S->have_v_in) {  // v_in = v_ext + V_H[rho0] + v_xc[rho0]
     if ((s = cs_hartree(c, S->rho, S->vh, work, stream)) != CS_OK) return s;
     if ((s = cs_lda_xc(c, S->rho, nullptr, S->vxc, stream)) != CS_OK) return s;
     k_sum3<<<grid_for(ng), 256, 0, st>>>(S->v_ext, S->vh, S->vxc, ng, S->v_in);
@@ -772,6 +785,8 @@ cs_status cs_scf_step(cs_scf* S, double* X, long long ld, double* theta, double*
   if ((s = cs_fermi_occupations(p.n_s, S->theta_h.data(), p.n_electrons, p.kT, S->occ_h.data(),
                                 &mu, &ent)) != CS_OK)
     return sfail(c, s, "cs_scf_step: Fermi level not found");
+  // the eigensolve has read the error word after v_in was made; rho is overwritten from here on
+  S->have_v_in = true;
   SCF_CUDA(c, cudaMemcpyAsync(S->occ_dev, S->occ_h.data(), p.n_s * 8, cudaMemcpyHostToDevice, st));
   if ((s = cs_density(c, p.n_s, X, ld, S->occ_dev, S->rho, work, stream)) != CS_OK) return s;
   if ((s = cs_hartree(c, S->rho, S->vh, work, stream)) != CS_OK) return s;
