@@ -317,21 +317,22 @@ cs_status cs_lobpcg(cs_ctx* ctx, int n_s, int n_want, double* X, long long ld, d
 cs_status cs_profile_begin(cs_ctx* ctx);
 cs_status cs_profile_end(cs_ctx* ctx, double* ms, long long* launches);
 
-/* H X like cs_apply_H (FP64 in FP64 arithmetic at every size, so that large blocks may differ from
- * cs_apply_H in the last bits), for callers that cannot allocate device memory when they call (for
- * example when another allocator already holds the free device memory, or when a loop must
- * not take the device-wide synchronisation of cudaMalloc/cudaFree). It needs no workspace:
- * its scratch is a 32 MiB array compiled into the library, present on every GPU that loads
- * the library until the process exits; it calls no allocation routine. The paper has no
- * counterpart; this is a deployment variant of the same H.X kernels.
+/* H X like cs_apply_H, by the same kernels and with the same bits, for callers that cannot
+ * allocate device memory when they call (for example when another allocator already holds the
+ * free device memory, or when a loop must not take the device-wide synchronisation of
+ * cudaMalloc/cudaFree). It needs no workspace: its scratch is a 32 MiB array compiled into the
+ * library, present on every GPU that loads the library until the process exits; it calls no
+ * allocation routine. The paper has no counterpart; this is a deployment variant of the same H.X
+ * kernels. FP64 blocks that do not fit the array with their intermediates run some states at a
+ * time.
  * Limits and rules: prec must be CS_FP64 or CS_FP32 (CS_ERR_ARG otherwise); N_r (lmax+1)^2
  * n_s x element size must be <= 32 MiB (else CS_ERR_ARG); no projectors (CS_ERR_STATE if
  * set); the first call on a device looks up the array's device address and keeps it, so make
  * that call before any stream capture on that device, and make no call on a device after a
  * cudaDeviceReset of it; all calls on a device share the array (it keeps the last call's
  * contents; nothing in it must start at zero), so calls that overlap on the GPU race and must
- * be serialised. The caller's current device is restored on return. Other arguments as
- * cs_apply_H without `work`. */
+ * be serialised. The caller's current device is restored on return. Other arguments, and expired
+ * device waits, as cs_apply_H without `work`. */
 cs_status cs_apply_H_noalloc(cs_ctx* ctx, int n_s, const void* X, void* HX, long long ld,
                              cs_precision prec, cs_stream stream);
 

@@ -24,8 +24,14 @@
 //     different host threads) race on it: serialise them.
 //   - Nothing in the array has to start at zero: the radial synthesis writes every
 //     element of G that the later kernels read.
+//   - FP64 blocks that cs_apply_H sends through the slice products take them here too, so that
+//     both calls return the same bits: in blocks of states whose G fills at most half the array,
+//     the other half holding the intermediates of some radial nodes at a time (so every block
+//     takes the path that cs_apply_H takes at its size). Their bounded waits report through the
+//     context's device error word, as in cs_apply_H.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -96,6 +102,52 @@ cs_status run(cs_ctx* c, int n_s, const T* X, T* HX, long long ld, T* G, cudaStr
   return CS_OK;
 }
 
+// States per pass of the slice products: G and its scales in one half of the array, at least one
+// radial node's intermediates in the other. Every basis that takes the slice products has room for
+// one state (63^2 harmonics, 448 nodes: 14.2 MB and 0.4 MB).
+int sliced_block(const cs::HostTables& H, int n_s) {
+  const size_t half = kScratchBytes / 2;
+  const size_t state = (size_t)H.n_r * H.L * H.L * 8 + cs::sliced_hx_fixed_bytes(H.n_r, 1);
+  const size_t node = cs::sliced_hx_node_bytes(H.L, H.n_theta, H.n_phi, 1);
+  const size_t fit = std::max<size_t>(1, std::min(half / (state + 256), half / node));
+  const int most = (int)std::min<size_t>(n_s, fit), passes = (n_s + most - 1) / most;
+  return (n_s + passes - 1) / passes;
+}
+
+cs_status run_sliced(cs_ctx* c, int n_s, const double* X, double* HX, long long ld, char* scratch,
+                     cudaStream_t st) {
+  const cs::HostTables& H = c->host;
+  const int per = sliced_block(H, n_s);
+  const size_t g = ((size_t)H.n_r * H.L * H.L * 8 * per + 255) & ~size_t(255);
+  const size_t fixed = g + cs::sliced_hx_fixed_bytes(H.n_r, per);
+  if (fixed + cs::sliced_hx_node_bytes(H.L, H.n_theta, H.n_phi, per) > kScratchBytes) {
+    c->err = "cs_apply_H_noalloc: the static scratch has no room for one radial node";
+    return CS_ERR_ARG;
+  }
+  for (int s0 = 0; s0 < n_s; s0 += per) {
+    const int n = std::min(per, n_s - s0);
+    cs::Epilogue<double> ep;
+    ep.mode = cs::EP_APPLY;
+    ep.out = HX + (size_t)s0 * ld;
+    ep.X = X + (size_t)s0 * ld;
+    ep.ld = ld;
+    ep.ld_out = ld;
+    ep.half_lambda = c->d64.half_lambda;
+    for (int stage = 0; stage < 3; ++stage) {
+      int nl = 0;
+      const cudaError_t e = cs::launch_sliced_hx(
+          H, c->sliced, n, X + (size_t)s0 * ld, ld, reinterpret_cast<double*>(scratch), ep,
+          scratch + g, c->dev_err, st, stage, &nl, kScratchBytes - fixed);
+      if (e != cudaSuccess) {
+        c->err = std::string("cs_apply_H_noalloc launch: ") + cudaGetErrorString(e);
+        return CS_ERR_CUDA;
+      }
+      c->launches += nl;
+    }
+  }
+  return CS_OK;
+}
+
 }  // namespace
 
 extern "C" cs_status cs_apply_H_noalloc(cs_ctx* c, int n_s, const void* X, void* HX,
@@ -140,7 +192,9 @@ extern "C" cs_status cs_apply_H_noalloc(cs_ctx* c, int n_s, const void* X, void*
   void* scratch = scratch_on_device(c->device, c->err);
   if (scratch) {
     cudaStream_t st = (cudaStream_t)stream;
-    r = prec == CS_FP64
+    r = prec == CS_FP64 && cs::use_sliced(c, n_s, false)
+            ? run_sliced(c, n_s, (const double*)X, (double*)HX, ld, (char*)scratch, st)
+        : prec == CS_FP64
             ? run<double>(c, n_s, (const double*)X, (double*)HX, ld, (double*)scratch, st)
             : run<float>(c, n_s, (const float*)X, (float*)HX, ld, (float*)scratch, st);
   }

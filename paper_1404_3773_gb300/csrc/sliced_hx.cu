@@ -1079,7 +1079,7 @@ int exp_above(double m) {  // 2^e >= m
 // Intermediates of one chunk of radial nodes. Larger chunks fill the last wave of each launch
 // better than smaller ones keep the intermediates in the 129 MB L2: 80-state H.X at lmax 30
 // 1.53 ms at 512 MB, 1.59 at 256, 1.74 at 128, 1.85 at 64.
-constexpr size_t kChunkBytes = (size_t)512 << 20;
+constexpr size_t kChunkBytes = kSlChunkBytes;
 constexpr int kMaxSB = 128;
 
 size_t al(size_t x) { return (x + 255) & ~size_t(255); }
@@ -1089,11 +1089,11 @@ size_t node_bytes(int L, int n_theta, int n_phi, int SB) {
   return (2 * NP * M2 + (size_t)n_theta * 4 * Q) * SB * 8 + (size_t)n_theta * SB * 12 + SB * 4;
 }
 
-void chunking(int L, int n_r, int n_theta, int n_phi, int S, int& SB, int& kc) {
+void chunking(int L, int n_r, int n_theta, int n_phi, int S, size_t bytes, int& SB, int& kc) {
   const int nblk = (S + kMaxSB - 1) / kMaxSB;
   SB = (S + nblk - 1) / nblk;
   const size_t nb = node_bytes(L, n_theta, n_phi, SB);
-  int most = (int)std::max<size_t>(1, kChunkBytes / nb);
+  int most = (int)std::max<size_t>(1, bytes / nb);
   const int nchunks = (n_r + most - 1) / most;
   kc = (n_r + nchunks - 1) / nchunks;
 }
@@ -1144,11 +1144,17 @@ bool sliced_hx_eligible(int L, int N, int n_r, int n_theta, int n_phi) {
 
 bool sliced_hx_enabled() { return getenv("CS_ANGULAR_KERNEL") == nullptr; }
 
+// What SlPlan takes beside the intermediates, and one node of them: the least it runs in.
+size_t sliced_hx_fixed_bytes(int n_r, int S) { return (size_t)n_r * S * 4 + 7 * 256; }
+size_t sliced_hx_node_bytes(int L, int n_theta, int n_phi, int S) {
+  return node_bytes(L, n_theta, n_phi, std::min(S, kMaxSB));
+}
+
 // An upper bound of what SlPlan takes that grows with S, so that a workspace sized for S states
 // serves every smaller block: at most n_r nodes, and at most kChunkBytes or one node.
 size_t sliced_hx_work_bytes(int L, int n_r, int n_theta, int n_phi, int S) {
   const size_t node = node_bytes(L, n_theta, n_phi, std::min(S, kMaxSB));
-  return std::min((size_t)n_r * node, kChunkBytes + node) + (size_t)n_r * S * 4 + 7 * 256;
+  return std::min((size_t)n_r * node, kChunkBytes + node) + sliced_hx_fixed_bytes(n_r, S);
 }
 
 void free_sliced_tables(SlicedTables& T) {
@@ -1245,11 +1251,11 @@ struct SlPlan {
   Geo g[6];
 
   SlPlan(const HostTables& H_, const SlicedTables& T_, int S, double* G, void* work, int* err,
-         cudaStream_t st_)
+         cudaStream_t st_, size_t bytes = kChunkBytes)
       : H(H_), T(T_), st(st_), L2(H_.L * H_.L), Np(H_.n_phi) {
     const int L = H.L, NP = (H.n_theta + 1) / 2, half = (L + 1) / 2;
     for (int op = 0; op < 6; ++op) g[op] = geo(op, L, H.N, H.n_r, H.n_theta, H.n_phi);
-    chunking(L, H.n_r, H.n_theta, H.n_phi, S, SBm, kcm);
+    chunking(L, H.n_r, H.n_theta, H.n_phi, S, bytes, SBm, kcm);
     for (int l = 0; l < L; ++l) rad_tiles += ((long long)(2 * l + 1) * S + kRows - 1) / kRows;
     char* p = static_cast<char*>(work);
     auto take = [&](size_t b) {
@@ -1370,8 +1376,8 @@ unsigned warp_grid(long long items) { return (unsigned)((items + 7) / 8); }
 
 cudaError_t launch_sliced_hx(const HostTables& H, const SlicedTables& T, int S, const double* X,
                              long long ld, double* G, const Epilogue<double>& ep, void* work,
-                             int* err, cudaStream_t st, int stage, int* launches) {
-  SlPlan p(H, T, S, G, work, err, st);
+                             int* err, cudaStream_t st, int stage, int* launches, size_t bytes) {
+  SlPlan p(H, T, S, G, work, err, st, bytes);
   SlArgs& a = p.a;
   cudaError_t e;
   if (stage == 0) {

@@ -26,7 +26,13 @@ struct SlicedTables {
 bool sliced_hx_eligible(int L, int N, int n_r, int n_theta, int n_phi);
 // CS_ANGULAR_KERNEL (any value) keeps the FMA kernels
 bool sliced_hx_enabled();
+// default size of the chunk intermediates
+constexpr size_t kSlChunkBytes = (size_t)512 << 20;
 size_t sliced_hx_work_bytes(int L, int n_r, int n_theta, int n_phi, int S);
+// A smaller workspace for S states: the fixed part and intermediates of at least one radial node.
+// The results do not depend on the split: every scale belongs to one state's row.
+size_t sliced_hx_fixed_bytes(int n_r, int S);
+size_t sliced_hx_node_bytes(int L, int n_theta, int n_phi, int S);
 // rad, theta: the FP64 device tables
 cudaError_t build_sliced_tables(const HostTables& H, const double* rad, const double* theta,
                                 SlicedTables& T);
@@ -34,10 +40,11 @@ void free_sliced_tables(SlicedTables& T);
 cudaError_t launch_sliced_wv(const SlicedTables& T, const double* wv, int rows, int n_phi,
                              cudaStream_t st);
 // stage 0: radial synthesis X -> G; 1: the angular block on G, in place; 2: radial analysis of G
-// with the epilogue. *launches receives the kernel count.
+// with the epilogue. *launches receives the kernel count. bytes: room for the chunk intermediates.
 cudaError_t launch_sliced_hx(const HostTables& H, const SlicedTables& T, int S, const double* X,
                              long long ld, double* G, const Epilogue<double>& ep, void* work,
-                             int* err, cudaStream_t st, int stage, int* launches);
+                             int* err, cudaStream_t st, int stage, int* launches,
+                             size_t bytes = kSlChunkBytes);
 
 // Grid values f[s][k][j][q] of S columns of X, or, with X null, of the radial synthesis in G.
 cudaError_t launch_sliced_grid(const HostTables& H, const SlicedTables& T, int S, const double* X,
