@@ -25,7 +25,7 @@ thread_local std::string g_init_error;
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Layout {
-  size_t G, Yalt, X32, Wkb, kbZ, HX, tmp, part, small, lanV, status, HXr, chw, oz, wd, sl, kbtc, wa,
+  size_t G, Yalt, X32, Wkb, kbZ, HX, tmp, small, lanV, status, HXr, chw, part, oz, wd, kbtc, wa, sl,
       total;
 };
 
@@ -52,10 +52,6 @@ Layout layout(const cs_ctx* c, int n_s, cs_precision prec) {
   o.kbZ = take(np ? d * ns * 8 : 0);
   o.HX = take(d * ns * 8);
   o.tmp = take(d * ns * 8);
-  size_t part = std::max(gram_partial_elems(T.d, n_s, n_s),
-                         gram_partial_elems(T.d, kMaxLanczos + 1, 1));
-  if (np) part = std::max(part, gram_partial_elems(T.d, (int)np, n_s));
-  o.part = take(part * 8);
   // small matrices: Gram / Rayleigh-Ritz matrix, rotation, and the eigensolver scratch
   // (8 m^2 + 3 m + 4 doubles), with m = max(n_s, Lanczos size)
   const size_t mm = std::max<size_t>(ns, kMaxLanczos + 2);
@@ -66,6 +62,13 @@ Layout layout(const cs_ctx* c, int n_s, cs_precision prec) {
   o.HXr = take(d * ns * 8);
   // weights s_i(theta_j) of the residual-form filter: FP64 table and one in the block type
   o.chw = take((size_t)(kMaxRitzDegree + 1) * ns * 16);
+  // From here on: what no FP64-class H X needs while its kernels run (the projector products, which
+  // do, come before them). The intermediates of the slice-product H X lie over it.
+  const size_t shared = off;
+  size_t part = std::max(gram_partial_elems(T.d, n_s, n_s),
+                         gram_partial_elems(T.d, kMaxLanczos + 1, 1));
+  if (np) part = std::max(part, gram_partial_elems(T.d, (int)np, n_s));
+  o.part = take(part * 8);
   // split operands and partial sums of the slice-product Gram matrices and rotations (and of
   // the FP64 projector pair, which takes the same arithmetic)
   size_t ozb = 0;
@@ -81,8 +84,6 @@ Layout layout(const cs_ctx* c, int n_s, cs_precision prec) {
   o.wd = take(angular_wide_df_eligible(T.L, T.n_theta, T.n_phi)
                   ? angular_wide_df_work_bytes(T.L, T.n_r, T.n_theta)
                   : 0);
-  // intermediates of the slice-product FP64 H.X (one chunk of radial nodes)
-  o.sl = take(c->sliced_ok ? sliced_hx_work_bytes(T.L, T.n_r, T.n_theta, T.n_phi, n_s) : 0);
   // last, so that every other offset is the same for both precisions
   auto is_f32 = [](cs_precision p) { return p == CS_FP32 || p == CS_MIXED_BF16; };
   const bool reduced = is_f32(prec) || is_f32(c->rr_prec);
@@ -95,7 +96,12 @@ Layout layout(const cs_ctx* c, int n_s, cs_precision prec) {
   o.wa = take(mixed && angular_wide_eligible(T.L, T.n_theta, T.n_phi)
                   ? angular_wide_work_bytes(T.L, T.n_r, T.n_theta, n_s)
                   : 0);
-  o.total = off;
+  // intermediates of the slice-product FP64 H.X (one chunk of radial nodes), over the slots above;
+  // whatever the precision, because a workspace for a reduced one also serves the FP64-class calls
+  o.sl = shared;
+  if (c->sliced_ok)
+    off = std::max(off, shared + sliced_hx_work_bytes(T.L, T.n_r, T.n_theta, T.n_phi, n_s));
+  o.total = al256(off);
   return o;
 }
 

@@ -55,7 +55,8 @@ struct ScfLayout {
   size_t alm;      // L^2 doubles (harmonic-term amplitudes)
   size_t G1;       // N_r L^2 doubles (Hartree radial synthesis)
   size_t partial;  // kDotBlocks x CS_GRID_INTEGRALS_MAX doubles
-  size_t slG, slw; // radial synthesis and intermediates of kSlChunk states (slice products)
+  size_t slG, slw; // radial synthesis and intermediates of kSlChunk states (slice products), over
+                   // trans and fgrid: neither is in use beside them
   size_t total;
 };
 
@@ -77,13 +78,18 @@ ScfLayout scf_layout(const cs_ctx* c) {
   const size_t L2 = (size_t)H.L * H.L;
   o.trans = take(tw);
   o.fgrid = take((size_t)n_grid(c) * CS_DENSITY_CHUNK * 8);
+  if (c->sliced_ok) {
+    const size_t end = off;
+    off = 0;
+    o.slG = take((size_t)H.n_r * L2 * kSlChunk * 8);
+    o.slw = take(sliced_hx_work_bytes(H.L, H.n_r, H.n_theta, H.n_phi, kSlChunk));
+    off = std::max(off, end);
+  }
   o.coef = take((size_t)H.d * 8);
   o.alm = take(L2 * 8);
   o.G1 = take((size_t)H.n_r * L2 * 8);
   // partials, results, device error word
   o.partial = take(((size_t)(kDotBlocks + 1) * CS_GRID_INTEGRALS_MAX + 1) * 8);
-  o.slG = take(c->sliced_ok ? (size_t)H.n_r * L2 * kSlChunk * 8 : 0);
-  o.slw = take(c->sliced_ok ? sliced_hx_work_bytes(H.L, H.n_r, H.n_theta, H.n_phi, kSlChunk) : 0);
   o.total = off;
   return o;
 }
