@@ -109,7 +109,7 @@ namespace cs {
 // meet: 0.130 / 0.122 ms at 7.4M (lmax 16, 16 states), 0.177 / 0.181 at 15M (lmax 23, 8),
 // 0.168 / 0.193 at 15M (lmax 16, 32), 0.254 / 0.336 at 44M (lmax 30, 8).
 inline bool use_sliced(const cs_ctx* c, int n_s, bool df) {
-  if (!c->sliced_ok || !sliced_hx_enabled()) return false;
+  if (!c->sliced_ok || !sliced_hx_enabled(df)) return false;
   const HostTables& H = c->host;
   const long long rows = (long long)H.n_r * H.n_theta * n_s;
   return rows * H.L * H.L >= 14000000 || (!df && rows >= 4096);

@@ -398,7 +398,8 @@ static cudaError_t launch_angular_st(const AngArgs<T>& a, int st, T* G, T* gout,
 // Which ANG_FULL kernel runs. FP32: the register-blocked kernel (angular_gm.cu) when its
 // tile fits in shared memory, else the row-pair kernel (angular_rp.cu); FP64: the row-pair
 // kernel; both fall back to the row-stream kernel above. CS_ANGULAR_KERNEL=gm|rp|rpN|stream
-// overrides the choice (N = tile variant), for tuning.
+// overrides the choice (N = tile variant), for tuning; gm and rp are FP32's and everyone's, so that
+// an FP64 call under gm keeps its default (see sliced_hx_enabled too).
 static int angular_choice(int& variant) {
   variant = -1;
   const char* e = getenv("CS_ANGULAR_KERNEL");

@@ -1142,7 +1142,15 @@ bool sliced_hx_eligible(int L, int N, int n_r, int n_theta, int n_phi) {
   return L <= 63 && N <= 448 && n_r <= 448 && (n_theta + 1) / 2 <= 64 && n_phi / 4 + 1 <= 64;
 }
 
-bool sliced_hx_enabled() { return getenv("CS_ANGULAR_KERNEL") == nullptr; }
+// CS_ANGULAR_KERNEL keeps the FMA kernels where it names one of them: stream, rp.. or fma; wide
+// names the three-pass blocks, of which FP64 has none. gm and tc choose among FP32 and mixed
+// kernels and, like the empty string, leave these calls alone.
+bool sliced_hx_enabled(bool df) {
+  const char* e = getenv("CS_ANGULAR_KERNEL");
+  if (!e) return true;
+  const bool fma = e[0] == 's' || (e[0] == 'r' && e[1] == 'p') || e[0] == 'f';
+  return !fma && !(df && e[0] == 'w');
+}
 
 // What SlPlan takes beside the intermediates, and one node of them: the least it runs in.
 size_t sliced_hx_fixed_bytes(int n_r, int S) { return (size_t)n_r * S * 4 + 7 * 256; }

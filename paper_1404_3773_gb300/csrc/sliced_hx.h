@@ -24,8 +24,8 @@ struct SlicedTables {
 // lmax <= 62, n_theta <= 128, n_phi <= 255 (64 table rows or K per class); N, n_r <= 448 (the
 // 64-bit sums of the radial products)
 bool sliced_hx_eligible(int L, int N, int n_r, int n_theta, int n_phi);
-// CS_ANGULAR_KERNEL (any value) keeps the FMA kernels
-bool sliced_hx_enabled();
+// whether CS_ANGULAR_KERNEL leaves them on (df: for a double-float call)
+bool sliced_hx_enabled(bool df);
 // default size of the chunk intermediates
 constexpr size_t kSlChunkBytes = (size_t)512 << 20;
 size_t sliced_hx_work_bytes(int L, int n_r, int n_theta, int n_phi, int S);
