@@ -122,12 +122,27 @@ def peak_word(peaks):
     return "fallback" if peaks.get("source") == "fallback" else "measured"
 
 
-def roofline_table(cs, w, d, n_s, prec, prof_ms, prof_n, steps, dense_prec):
+def split_sliced(names, prof_ms, prof_n, sliced):
+    """(name, ms, launches) per profile class, with what ran as slice products on the tensor cores
+    (FP64 H.X, and double-float H.X that takes the same products) in classes of its own."""
+    if sliced is None:
+        sliced = ([0.0] * len(names), [0] * len(names))
+    out, own = [], {}
+    for i, name in enumerate(names):
+        out.append((name, prof_ms[i] - sliced[0][i], prof_n[i] - sliced[1][i]))
+        if sliced[1][i]:
+            fam = name[:-len("_df64")] if name.endswith("_df64") else name
+            ms, n = own.get(fam, (0.0, 0))
+            own[fam] = (ms + sliced[0][i], n + sliced[1][i])
+    return out + [(fam + "_sliced", ms, n) for fam, (ms, n) in own.items()]
+
+
+def roofline_table(cs, w, d, n_s, prec, prof_ms, prof_n, steps, dense_prec, sliced=None):
     """Per kernel class: launches, share of device time, algorithmic TFLOP/s and the fraction
     of the pipe that bounds it; the dominant class becomes the `roofline` object. The dense
     class (Gram matrices and rotations of CholQR2 and Rayleigh-Ritz, factor, eigensolve) is
     rated against the pipe its Gram matrices and rotations run on: FP64, or the FP32 pipe in
-    double-float."""
+    double-float. `sliced`: what of the classes ran as slice products (cs_profile_sliced)."""
     from paper_1404_3773_gb300 import CS_DF64, CS_FP64_SLICED, CS_MIXED_BF16
     names = cs.profile_class_names()
     af = algorithmic_flops(w, n_s)
@@ -135,20 +150,20 @@ def roofline_table(cs, w, d, n_s, prec, prof_ms, prof_n, steps, dense_prec):
     bf16 = peaks.get("bf16_tflops_sustained")
     total = max(1e-9, sum(prof_ms))
     classes = {}
-    for i, name in enumerate(names):
-        if prof_n[i] == 0:
+    for name, cls_ms, cls_n in split_sliced(names, prof_ms, prof_n, sliced):
+        if cls_n == 0:
             continue
-        kind = "f32" if name.endswith("_f32") else ("df64" if name.endswith("_df64") else "f64")
+        kind = next((k for k in ("f32", "df64", "sliced") if name.endswith("_" + k)), "f64")
         fam = name.rsplit("_", 1)[0] if kind != "f64" else name
         f32 = kind == "f32"
-        per_ms = prof_ms[i] / prof_n[i]
+        per_ms = cls_ms / cls_n
         mixed_ang = f32 and prec == CS_MIXED_BF16 and fam == "angular"
         if mixed_ang:
             flops = af["angular_fp32_pipe"]
         elif fam in ("radial_synth", "radial_anal", "angular"):
             flops = af[fam]
         elif fam == "dense":
-            flops = dense_flops(d, n_s) / max(1.0, prof_n[i] / steps)
+            flops = dense_flops(d, n_s) / max(1.0, cls_n / steps)
         else:
             flops = None
         if f32 and prec == CS_MIXED_BF16 and fam.startswith("radial") and bf16:
@@ -159,6 +174,11 @@ def roofline_table(cs, w, d, n_s, prec, prof_ms, prof_n, steps, dense_prec):
                 "on the FP32 pipe (the phi transforms run on tcgen05 and are not counted)")
         elif f32:
             bound, peak, src = "alu", FP32_PEAK_TFLOPS, "152 SMs x 128 FP32 lanes x 2 x 2.07 GHz"
+        elif kind == "sliced" and bf16:
+            # each FP64 product is 34 BF16 digit products (7 digits, diagonals 0 .. 7)
+            bound, peak, src = "tensor", bf16 / 34.0, (
+                f"{peak_word(peaks)} bf16 sustained / 34 (FP64-equivalent rate of the digit "
+                "products; splitting and joining on the integer pipe bounds these kernels first)")
         elif fam == "dense" and dense_prec == CS_FP64_SLICED and bf16:
             # each FP64 product is 36 BF16 slice products (8 digits, pairs k + l <= 7)
             bound, peak, src = "tensor", bf16 / 36.0, (
@@ -170,8 +190,8 @@ def roofline_table(cs, w, d, n_s, prec, prof_ms, prof_n, steps, dense_prec):
         else:
             bound, peak, src = "alu", FP64_PEAK_TFLOPS, "FP64 nominal 1.25 TFLOP/s (GB300)"
         ach = flops / (per_ms / 1e3) / 1e12 if flops else None
-        classes[name] = {"launches": int(prof_n[i]), "ms": round(prof_ms[i], 4),
-                         "share": round(prof_ms[i] / total, 4),
+        classes[name] = {"launches": int(cls_n), "ms": round(cls_ms, 4),
+                         "share": round(cls_ms / total, 4),
                          "avg_launch_ms": round(per_ms, 5),
                          "flops_per_launch": flops,
                          "achieved": round(ach, 4) if ach else None,
@@ -343,6 +363,7 @@ def run_ours(args):
         total_ms += e0.elapsed_time(e1)
     torch.cuda.synchronize()
     prof_ms, prof_n = cs.cs_profile_end(ctx)
+    prof_sliced = cs.cs_profile_sliced(ctx)
     if world > 1:
         total_ms = reduce_max_time(total_ms, world, device=dev)
         torch.distributed.barrier()
@@ -464,7 +485,7 @@ def run_ours(args):
 
     # ---- roofline of the dominant kernel class (device time measured live above)
     roofline, classes = roofline_table(cs, w, d, n_s, prec, prof_ms, prof_n, args.steps,
-                                       dense_prec)
+                                       dense_prec, prof_sliced)
     # the FP32 / FP64 FMA rates measured on this device, beside the nominal unit-count peaks
     alu = None
     try:
@@ -541,20 +562,28 @@ def step_breakdown(classes, steps, degree, ms_per_step, prec, rr_prec):
     """Per ChFSI iteration: the filter pass (degree H.X with the recurrence), one Chebyshev
     step, the Rayleigh-Ritz H.X and the dense part, from the per-class device times; and the
     step's roofline time, the sum over classes of algorithmic flops / the bounding pipe's peak
-    (every class here is ALU-bound: its bytes / HBM bandwidth is far smaller)."""
+    (every class here is bound by a pipe: its bytes / HBM bandwidth is far smaller). The
+    "_sliced" classes hold the FP64-class products, of the filter or of the Rayleigh-Ritz H.X."""
     from paper_1404_3773_gb300 import CS_FP64, CS_FP32, CS_MIXED_BF16, CS_DF64
     sfx = {CS_FP64: "", CS_FP32: "_f32", CS_MIXED_BF16: "_f32", CS_DF64: "_df64"}
     fams = ("radial_synth", "angular", "radial_anal", "kb")
 
-    def hx_ms(suffix):
-        return sum(classes[f + suffix]["ms"] for f in fams if f + suffix in classes) / steps
+    def hx_ms(*suffixes):
+        return sum(classes[f + s]["ms"] for s in suffixes for f in fams
+                   if f + s in classes) / steps
 
-    filt = hx_ms(sfx[prec])
-    if sfx[rr_prec] == sfx[prec]:  # filter and Rayleigh-Ritz applies share the classes
+    f64_class = (CS_FP64, CS_DF64)
+    if prec in f64_class and rr_prec in f64_class and "angular_sliced" in classes:
+        filt = hx_ms("", "_df64", "_sliced")
+        rr = filt / (degree + 1)  # both applies share the slice-product classes
+        filt -= rr
+    elif sfx[rr_prec] == sfx[prec]:  # filter and Rayleigh-Ritz applies share the classes
+        filt = hx_ms(sfx[prec])
         rr = filt / (degree + 1)
         filt -= rr
     else:
-        rr = hx_ms(sfx[rr_prec])
+        filt = hx_ms(sfx[prec], *["_sliced"] * (prec in f64_class))
+        rr = hx_ms(sfx[rr_prec], *["_sliced"] * (rr_prec in f64_class))
     dense = classes["dense"]["ms"] / steps if "dense" in classes else 0.0
     roof = 0.0
     for c in classes.values():
@@ -1210,7 +1239,9 @@ def at_scale_chfsi_measure(dev, chunk=128, timed_iters=2, cpu_seconds=10.0):
         times.append(e0.elapsed_time(e1))
         hist.append(float(resid[:w.n_want].max()))
     pms, pn = cs.cs_profile_end(ctx)
-    names = cs.profile_class_names()
+    parts = split_sliced(cs.profile_class_names(), pms, pn, cs.cs_profile_sliced(ctx))
+    names = [nm for nm, _, _ in parts]
+    pms, pn = [t for _, t, _ in parts], [n for _, _, n in parts]
     ms = sum(times) / len(times)
     hx_per_iter = degree  # degree - 1 filter products + the Rayleigh-Ritz one, per state
     applies = hx_per_iter * n_s

@@ -316,6 +316,9 @@ cs_status cs_lobpcg(cs_ctx* ctx, int n_s, int n_want, double* X, long long ld, d
 #define CS_PROFILE_CLASSES 15
 cs_status cs_profile_begin(cs_ctx* ctx);
 cs_status cs_profile_end(cs_ctx* ctx, double* ms, long long* launches);
+/* Of the classes of the last cs_profile_end, the part that ran as slice products on the tensor
+ * cores (CS_FP64, and CS_DF64 calls that take them): arrays as there. */
+cs_status cs_profile_sliced(const cs_ctx* ctx, double* ms, long long* launches);
 
 /* H X like cs_apply_H, by the same kernels and with the same bits, for callers that cannot
  * allocate device memory when they call (for example when another allocator already holds the

@@ -23,7 +23,8 @@ __all__ = [
     "cs_kinetic", "cs_bessel_zeros", "cs_set_potential", "cs_set_projectors",
     "cs_forward_transform", "cs_inverse_transform", "cs_workspace_bytes", "cs_apply_H",
     "cs_cheb_filter", "cs_cholqr", "cs_rayleigh_ritz", "cs_lanczos_bound", "cs_chfsi",
-    "cs_chfsi_step", "cs_cheb_filter_ritz", "cs_chfsi_step_ritz", "cs_profile_begin", "cs_profile_end", "cs_apply_H_noalloc",
+    "cs_chfsi_step", "cs_cheb_filter_ritz", "cs_chfsi_step_ritz", "cs_profile_begin", "cs_profile_end",
+    "cs_profile_sliced", "cs_apply_H_noalloc",
     "cs_set_rr_precision", "cs_set_dense_precision", "cs_dense_gram", "cs_dense_rotate",
     "cs_device_error", "Batch", "cs_batch_create", "cs_batch_free", "cs_batch_workspace_bytes",
     "cs_batch_cheb_filter", "cs_batch_tune", "cs_batch_tune_times", "cs_batch_set_variant",
@@ -122,6 +123,7 @@ _SIGS = {
     "cs_profile_begin": (_i, [_vp]),
     "cs_device_error": (_i, [_vp, ctypes.POINTER(_i)]),
     "cs_profile_end": (_i, [_vp, _dp, ctypes.POINTER(_ll)]),
+    "cs_profile_sliced": (_i, [_vp, _dp, ctypes.POINTER(_ll)]),
     "cs_set_rr_precision": (_i, [_vp, _i]),
     "cs_set_dense_precision": (_i, [_vp, _i]),
     "cs_dense_gram": (_i, [_vp, _i, _i, _vp, _ll, _vp, _ll, _vp, _ll, _vp, _vp]),
@@ -522,6 +524,14 @@ def cs_profile_end(ctx: Context):
     ms = (ctypes.c_double * PROFILE_CLASSES)()
     n = (_ll * PROFILE_CLASSES)()
     ctx.check(_lib.cs_profile_end(ctx.handle, ms, n))
+    return list(ms), list(n)
+
+
+def cs_profile_sliced(ctx: Context):
+    """(ms, launches) per class of the last cs_profile_end that ran as slice products."""
+    ms = (ctypes.c_double * PROFILE_CLASSES)()
+    n = (_ll * PROFILE_CLASSES)()
+    ctx.check(_lib.cs_profile_sliced(ctx.handle, ms, n))
     return list(ms), list(n)
 
 

@@ -163,6 +163,7 @@ struct ProfScope {
   } while (0)
 #define CS_LAUNCH(ctx, nk, expr) CS_LAUNCH_CLS(ctx, 3, nk, expr)
 constexpr int kProfFamilies = 5;  // classes per arithmetic (see cs_ctx::prof)
+constexpr int kProfSliced = 1 << 8;  // added to a record's class: a slice product
 template <typename T>
 constexpr int prof_cls(int family) {
   return family + (std::is_same<T, float>::value ? kProfFamilies
@@ -312,7 +313,7 @@ cs_status hx_core(cs_ctx* c, int n_s, const T* X, long long ldx, T* out, long lo
       const int base = as_df ? prof_cls<df64>(0) : prof_cls<T>(0);
       for (int stage = 0; stage < 3; ++stage) {
         int nl = 0;
-        CS_LAUNCH_CLS(c, base + stage, nl,
+        CS_LAUNCH_CLS(c, kProfSliced + base + stage, nl,
                       launch_sliced_hx(H, c->sliced, n_s, X, ldx, G, ep, work + lay.sl, c->dev_err,
                                        st, stage, &nl));
       }
@@ -1284,22 +1285,34 @@ cs_status cs_profile_end(cs_ctx* c, double* ms, long long* launches) {
   if (s != CS_OK) return s;
   if (!ms || !launches) return fail(c, CS_ERR_ARG, "NULL output");
   for (int i = 0; i < CS_PROFILE_CLASSES; ++i) {
-    ms[i] = 0.0;
-    launches[i] = 0;
+    ms[i] = c->prof_sliced_ms[i] = 0.0;
+    launches[i] = c->prof_sliced_n[i] = 0;
   }
   for (auto& r : c->prof_recs) {
     CS_CHECK_CUDA(c, cudaEventSynchronize(r.b));
     float t = 0.f;
     CS_CHECK_CUDA(c, cudaEventElapsedTime(&t, r.a, r.b));
-    if (r.cls >= 0 && r.cls < CS_PROFILE_CLASSES) {
-      ms[r.cls] += t;
-      launches[r.cls] += 1;
+    const int cls = r.cls & (kProfSliced - 1);
+    if (cls < CS_PROFILE_CLASSES) {
+      ms[cls] += t;
+      launches[cls] += 1;
+      if (r.cls & kProfSliced) {
+        c->prof_sliced_ms[cls] += t;
+        c->prof_sliced_n[cls] += 1;
+      }
     }
     c->event_pool.push_back(r.a);
     c->event_pool.push_back(r.b);
   }
   c->prof_recs.clear();
   c->prof = false;
+  return CS_OK;
+}
+
+cs_status cs_profile_sliced(const cs_ctx* c, double* ms, long long* launches) {
+  if (!c || !ms || !launches) return CS_ERR_ARG;
+  std::copy(c->prof_sliced_ms, c->prof_sliced_ms + CS_PROFILE_CLASSES, ms);
+  std::copy(c->prof_sliced_n, c->prof_sliced_n + CS_PROFILE_CLASSES, launches);
   return CS_OK;
 }
 

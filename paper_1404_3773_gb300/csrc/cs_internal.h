@@ -94,6 +94,9 @@ struct cs_ctx {
     cudaEvent_t a, b;
   };
   std::vector<ProfRec> prof_recs;
+  // of the last cs_profile_end: what ran as slice products (cs_profile_sliced)
+  double prof_sliced_ms[CS_PROFILE_CLASSES] = {};
+  long long prof_sliced_n[CS_PROFILE_CLASSES] = {};
   std::vector<cudaEvent_t> event_pool;
 };
 

@@ -36,3 +36,26 @@ def test_only_values_that_name_an_fma_kernel_switch_the_slices_off(value, monkey
     # the double-float call converts in and out around its own kernels
     assert (ndf == n_slices and torch.equal(b, ref)) != (FMA_FP64[value] or value == "wide")
     assert torch.equal(a, ref) or FMA_FP64[value]
+
+
+def test_profile_tells_the_slice_products_apart(monkeypatch):
+    torch, cs = need_gpu()
+    ctx = make_ctx(W1)
+    X = to_dev(W1.x_block())
+    out = torch.zeros_like(X)
+    names = cs.profile_class_names()
+
+    def profile(prec):
+        cs.cs_profile_begin(ctx)
+        cs.cs_apply_H(ctx, X, out, prec)
+        ms, n = cs.cs_profile_end(ctx)
+        sms, sn = cs.cs_profile_sliced(ctx)
+        assert all(0.0 <= b <= a for a, b in zip(ms, sms)) and len(names) == len(sn) == len(n)
+        return [{k: v for k, v in zip(names, x) if v} for x in (n, sn)]
+
+    monkeypatch.delenv("CS_ANGULAR_KERNEL", raising=False)
+    fams = ("radial_synth", "angular", "radial_anal")
+    assert profile(cs.CS_FP64) == [dict.fromkeys(fams, 1)] * 2
+    assert profile(cs.CS_DF64) == [{f + "_df64": 1 for f in fams}] * 2
+    monkeypatch.setenv("CS_ANGULAR_KERNEL", "fma")
+    assert profile(cs.CS_FP64) == [dict.fromkeys(fams, 1), {}]
