@@ -1,7 +1,7 @@
 // Dense FP64 pieces of the ChFSI iteration (Sec. 3.2.1): Gram matrices and block
 // rotations for Cholesky-QR (Sec. 3.1.1: Cholesky after column scaling) and Rayleigh-
-// Ritz, a one-CTA parallel cyclic Jacobi eigensolver for the projected matrix, residual
-// norms, conversions and small vector helpers.
+// Ritz, the symmetric eigensolver of the projected matrix (Householder tridiagonalisation, bisection
+// with inverse iteration, refinement in FP64), residual norms, conversions and small vector helpers.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -1305,7 +1305,10 @@ __global__ void k_ns_factor(const double* __restrict__ G, int n, double* __restr
   M[e] = (i == j ? 1.5 : 0.0) - 0.5 * G[e];
 }
 
-// Ep = I + E (n x n), grid over elements
+// Ep = I + E (n x n), grid over elements. V^T (A V) is symmetric only to the rounding of its products,
+// about 2^-53 |A|, which the division raises to 2^-53 |A| / gap. From the mean of S_ij and S_ji it
+// goes into E antisymmetrically, a rotation, and the vectors stay orthonormal: levels 1e-5 |A| apart
+// were 2e-12 off before (4e-12 with a third Newton-Schulz step).
 __global__ void k_oa_update(const double* __restrict__ S, const double* __restrict__ G, int n,
                             const double* __restrict__ lam, const double* __restrict__ scal,
                             double* __restrict__ Ep) {
@@ -1317,7 +1320,7 @@ __global__ void k_oa_update(const double* __restrict__ S, const double* __restri
   if (i == j) {
     v = 0.5 * r;
   } else {
-    const double num = S[e] + lam[j] * r;
+    const double num = 0.5 * (S[e] + S[j + (size_t)i * n]) + lam[j] * r;
     const double dl = lam[j] - lam[i];
     const double lim = fmax(scal[0], 1e3 * fabs(num));
     v = (fabs(dl) > lim) ? num / dl : 0.5 * r;
@@ -1849,7 +1852,7 @@ cudaError_t launch_sym_eig(const double* A, int n, double* theta, double* V, dou
     // refinement); status as the one-CTA solver's
     if ((e = le_stage(A, n, P, Ep, V0, status, stream)) != cudaSuccess) return e;
   }
-  // 2. orthonormalise to FP64 precision (Newton-Schulz), then refine in FP64. The 25 n x n
+  // 2. orthonormalise to FP64 precision (Newton-Schulz), then refine in FP64. The 23 n x n
   // products take the FP64 pipe (small_gemm) or, for large n when the caller hands over a
   // slice-product workspace, the exact slice products on the tensor cores: at n = 880 one
   // FP64-pipe product is about 1.1 ms at the pipe's peak
@@ -1876,7 +1879,10 @@ cudaError_t launch_sym_eig(const double* A, int n, double* theta, double* V, dou
   };
   double* Vc = V0;
   double* Vn = V1;
-  // FP32 vectors are orthonormal to 1e-6: two steps square that twice, below FP64's rounding
+  // Members of one cluster leave the FP32 stage orthonormal to 1e-6, but vectors of levels just
+  // outside the cluster width of 1e-5 |T| may overlap by eps |T| / gap, about 6e-3. Two steps
+  // (error -> 3/4 error^2) take that to 5e-10, and the refinement, which corrects V^T V as it goes,
+  // squares it four times more: levels 1.2e-5 to 1e-4 of the range apart end 2e-15 off at 80 states.
   for (int it = 0; it < 2; ++it) {
     if ((e = prod(true, Vc, Vc, G)) != cudaSuccess) return e;   // G = V^T V
     k_ns_factor<<<(unsigned)((n2 + 255) / 256), 256, 0, stream>>>(G, n, Ep);
