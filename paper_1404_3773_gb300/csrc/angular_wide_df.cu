@@ -18,6 +18,7 @@
 // as it is loaded.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdlib>
 #include <type_traits>
@@ -419,7 +420,16 @@ cudaError_t launch_angular_wide_df(const AngArgs<df64>& a, df64* G, df64* FA,
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return e;
   const size_t b1 = df_l1_elems(s) * sizeof(df64), b2 = df_l2_elems(s) * sizeof(df64);
-  const bool wide = df_p_wide_elems(s) * sizeof(df64) <= 227 * 1024;
+  // The table as broadcast pairs where it leaves as many CTAs on an SM as the table of values does
+  // (two at most, by registers): it saves instructions, but a lost CTA costs more. 128 states, 24
+  // radial nodes, lmax 60: at n_phi 180, one CTA either way, 2.59 ms with pairs (2.97 for values
+  // without packed instructions); at n_phi 124, where pairs leave one CTA of two, 2.29 with pairs
+  // and 1.96 with values (2.19 without packed instructions).
+  auto ctas = [](size_t elems) {
+    return std::min<size_t>(2, (228 * 1024) / (elems * sizeof(df64) + 1024));
+  };
+  const bool wide = df_p_wide_elems(s) * sizeof(df64) <= 227 * 1024 &&
+                    ctas(df_p_wide_elems(s)) >= ctas(df_p_elems(s));
   const size_t bp = (wide ? df_p_wide_elems(s) : df_p_elems(s)) * sizeof(df64);
   const auto phi = wide ? k_phi_df<true> : k_phi_df<false>;
   if ((e = cudaFuncSetAttribute(k_leg_synth_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
