@@ -194,6 +194,7 @@ struct MacAcc {
   __device__ __forceinline__ void set(C x) { v = x; }
   __device__ __forceinline__ void add_prod(C a, C b) { v = fma(a, b, v); }
   __device__ __forceinline__ C value() const { return v; }
+  __device__ __forceinline__ void renormalise() {}
 };
 template <>
 struct MacAcc<df64> {
@@ -204,6 +205,7 @@ struct MacAcc<df64> {
   }
   __device__ __forceinline__ void add_prod(df64 x, df64 y) { a.add_prod(x, y); }
   __device__ __forceinline__ df64 value() const { return a.value(); }
+  __device__ __forceinline__ void renormalise() { set(a.value()); }
 };
 
 }  // namespace cs

@@ -55,7 +55,8 @@ __device__ __forceinline__ double out_val(df64 v) { return v.to_double(); }
 
 // F: storage type of A, B and the partials; C: arithmetic (F, or df64 for F = double).
 // SYM (A and B are one block, one tile): only the 16 x 16 sub-blocks on and above the diagonal,
-// U (U + 1) / 2 of U^2; k_gram_reduce mirrors them.
+// U (U + 1) / 2 of U^2; k_gram_reduce mirrors them. A single sub-block is its own mirror image: both
+// of its triangles take the same products, in the same order of factors.
 template <typename F, typename C, int U, bool SYM>
 __global__ void __launch_bounds__(256) k_gram_partial(const F* __restrict__ A, long long lda,
                                                        const F* __restrict__ B,
@@ -84,15 +85,22 @@ __global__ void __launch_bounds__(256) k_gram_partial(const F* __restrict__ A, l
     for (int rr = 0; rr < GK; ++rr) {
       C a[U], b[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) a[u] = As[rr][tx + 16 * u];
+      for (int u = 0; u < U; ++u) a[u] = As[rr][(SYM && U == 1 ? min(tx, ty) : tx) + 16 * u];
 #pragma unroll
-      for (int v = 0; v < U; ++v) b[v] = SYM ? As[rr][ty + 16 * v] : Bs[rr][ty + 16 * v];
+      for (int v = 0; v < U; ++v)
+        b[v] = SYM ? As[rr][(U == 1 ? max(tx, ty) : ty) + 16 * v] : Bs[rr][ty + 16 * v];
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int v = SYM ? u : 0; v < U; ++v) acc[u][v].add_prod(a[u], b[v]);
     }
     __syncthreads();
+    // double-float: the trailing parts go into the leading ones every 16 rows, before their own
+    // rounding counts (A^T B of 80 columns, d = 46128: 6.7e-15 without, 2.9e-15 with; 3 % of the time)
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int v = SYM ? u : 0; v < U; ++v) acc[u][v].renormalise();
   }
   F* P = partial + (size_t)chunk * na * nb;
 #pragma unroll
@@ -104,23 +112,21 @@ __global__ void __launch_bounds__(256) k_gram_partial(const F* __restrict__ A, l
     }
 }
 
-// The double-float Gram tile on packed FP32 instructions: a thread keeps two sums per entry, over
-// the even and the odd rows, so that a pair of neighbouring rows is one operand pair as it lies in
-// shared memory ([column][row], leading and trailing parts apart). d = 46128, 80 columns: X^T X
-// 0.204 ms in the scalar form (0.112 with the sub-blocks below the diagonal left out).
-template <int U, bool SYM>
+// The double-float X^T X tile on packed FP32 instructions (one tile, the sub-blocks on and above the
+// diagonal): a thread keeps two sums per entry, over the even and the odd rows, so that a pair of
+// neighbouring rows is one operand pair as it lies in shared memory ([column][row], leading and
+// trailing parts apart). d = 46128, 80 columns: 0.109 ms, where all sub-blocks take 0.173 in the
+// scalar form. The full square stays scalar: there the second half's sums cost more registers than
+// the packing saves in issue (A^T B at 80 columns 0.211 against 0.196 ms, at 128 0.658 / 0.454).
+template <int U>
 __global__ void __launch_bounds__(256) k_gram_partial_df(const double* __restrict__ A,
-                                                         long long lda,
-                                                         const double* __restrict__ B,
-                                                         long long ldb, long long d, int na,
-                                                         int nb, long long rows,
+                                                         long long lda, long long d, int n,
+                                                         long long rows,
                                                          double* __restrict__ partial) {
   constexpr int T = 16 * U, P = GK + 2;
-  const int i0 = blockIdx.x * T, j0 = blockIdx.y * T;
   const long long r0 = (long long)blockIdx.z * rows;
   const long long r1 = min(d, r0 + rows);
   __shared__ __align__(8) float Ah[T][P], Al[T][P];
-  __shared__ __align__(8) float Bh[SYM ? 1 : T][P], Bl[SYM ? 1 : T][P];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   df64acc2 acc[U][U];
   for (long long rb = r0; rb < r1; rb += GK) {
@@ -128,14 +134,9 @@ __global__ void __launch_bounds__(256) k_gram_partial_df(const double* __restric
     for (int u = 0; u < U; ++u) {  // GK T values, 256 threads
       const int rr = tx, cc = ty + 16 * u;
       const long long r = rb + rr;
-      const df64 x((r < r1 && i0 + cc < na) ? A[r + (long long)(i0 + cc) * lda] : 0.0);
+      const df64 x((r < r1 && cc < n) ? A[r + (long long)cc * lda] : 0.0);
       Ah[cc][rr] = x.hi;
       Al[cc][rr] = x.lo;
-      if (!SYM) {
-        const df64 y((r < r1 && j0 + cc < nb) ? B[r + (long long)(j0 + cc) * ldb] : 0.0);
-        Bh[cc][rr] = y.hi;
-        Bl[cc][rr] = y.lo;
-      }
     }
     __syncthreads();
 #pragma unroll 2
@@ -143,8 +144,8 @@ __global__ void __launch_bounds__(256) k_gram_partial_df(const double* __restric
       float2 bh[U], bl[U];
 #pragma unroll
       for (int v = 0; v < U; ++v) {
-        bh[v] = *reinterpret_cast<const float2*>(&(SYM ? Ah : Bh)[ty + 16 * v][rr]);
-        bl[v] = *reinterpret_cast<const float2*>(&(SYM ? Al : Bl)[ty + 16 * v][rr]);
+        bh[v] = *reinterpret_cast<const float2*>(&Ah[ty + 16 * v][rr]);
+        bl[v] = *reinterpret_cast<const float2*>(&Al[ty + 16 * v][rr]);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -152,34 +153,37 @@ __global__ void __launch_bounds__(256) k_gram_partial_df(const double* __restric
         const float2 al = *reinterpret_cast<const float2*>(&Al[tx + 16 * u][rr]);
         const float2 nah = make_float2(-ah.x, -ah.y);
 #pragma unroll
-        for (int v = SYM ? u : 0; v < U; ++v) acc[u][v].add_prod(ah, nah, al, bh[v], bl[v]);
+        for (int v = u; v < U; ++v) acc[u][v].add_prod(ah, nah, al, bh[v], bl[v]);
       }
     }
     __syncthreads();
   }
-  double* Pt = partial + (size_t)blockIdx.z * na * nb;
+  double* Pt = partial + (size_t)blockIdx.z * n * n;
 #pragma unroll
   for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int v = SYM ? u : 0; v < U; ++v) {
-      const int i = i0 + tx + 16 * u, j = j0 + ty + 16 * v;
-      if (i < na && j < nb)
-        Pt[i + (size_t)j * na] = (acc[u][v].value(0) + acc[u][v].value(1)).to_double();
+    for (int v = u; v < U; ++v) {
+      const int i = tx + 16 * u, j = ty + 16 * v;
+      if (i < n && j < n)
+        Pt[i + (size_t)j * n] = (acc[u][v].value(0) + acc[u][v].value(1)).to_double();
     }
 }
 
-// 32 elements x 8 chunk slices per 256-thread block; slices summed in a fixed order; sym: the
+// 32 elements x 8 chunk slices per 256-thread block; slices summed in a fixed order; SYM: the
 // entries below the diagonal from those above
-template <typename F>
+template <typename F, bool SYM>
 __global__ void k_gram_reduce(const F* __restrict__ partial, int chunks, int na, int nb,
-                              F* __restrict__ C, int ldc, int sym) {
+                              F* __restrict__ C, int ldc) {
   __shared__ F red[8][33];
   const int el = threadIdx.x & 31, sl = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + el;
   const int E = na * nb;
   F s = F(0);
-  const int ei = e % na, ej = e / na;
-  const int src = sym && ei > ej ? ej + ei * na : e;
+  int src = e;
+  if (SYM) {
+    const int ei = e % na, ej = e / na;
+    if (ei > ej) src = ej + ei * na;
+  }
   if (e < E)
     for (int c = sl; c < chunks; c += 8) s += partial[(size_t)c * E + src];
   red[sl][el] = s;
@@ -203,14 +207,13 @@ static cudaError_t gram_impl(const F* A, long long lda, const F* B, long long ld
   const bool sym = A == B && lda == ldb && na == nb && ta == 1;
 #define CS_GRAM_CASE(UV)                                                                        \
   case UV:                                                                                      \
-    if constexpr (std::is_same<C, df64>::value && UV < 6) {                                     \
-      if (sym)                                                                                  \
-        k_gram_partial_df<UV, true><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows,  \
-                                                              partial);                         \
-      else                                                                                      \
-        k_gram_partial_df<UV, false><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, \
-                                                               partial);                        \
-    } else if (sym)                                                                                    \
+    if constexpr (std::is_same<C, df64>::value && UV > 1 && UV < 6) {                           \
+      if (sym) {                                                                                \
+        k_gram_partial_df<UV><<<grid, 256, 0, stream>>>(A, lda, d, na, rows, partial);          \
+        break;                                                                                  \
+      }                                                                                         \
+    }                                                                                           \
+    if (sym)                                                                                    \
       k_gram_partial<F, C, UV, true><<<grid, 256, 0, stream>>>(A, lda, B, ldb, d, na, nb, rows, \
                                                                partial);                        \
     else                                                                                        \
@@ -228,8 +231,11 @@ static cudaError_t gram_impl(const F* A, long long lda, const F* B, long long ld
   }
 #undef CS_GRAM_CASE
   int tot = na * nb;
-  k_gram_reduce<F><<<(tot + 31) / 32, 256, 0, stream>>>(partial, chunks, na, nb, Cout, ldc,
-                                                        sym ? 1 : 0);
+  if (sym && u > 1)
+    k_gram_reduce<F, true><<<(tot + 31) / 32, 256, 0, stream>>>(partial, chunks, na, nb, Cout, ldc);
+  else
+    k_gram_reduce<F, false><<<(tot + 31) / 32, 256, 0, stream>>>(partial, chunks, na, nb, Cout,
+                                                                 ldc);
   return cudaGetLastError();
 }
 
@@ -247,8 +253,8 @@ cudaError_t launch_gram_df(const double* A, long long lda, const double* B, long
 
 // ------------------------------------------------------------------ C = alpha A Q + beta C
 // 64 rows x (16U) columns per CTA; U from n so that 80 states are one column tile.
-// UPPER: Q is upper triangular with zeros stored below its diagonal, so a step of 16 rows k of Q
-// meets only the column groups of 16 that reach it (15 of 25 at 80 columns).
+// UPPER: Q is upper triangular with zeros stored below its diagonal, so a column tile ends at its last
+// column's row.
 template <typename F, typename Cm, int U, bool UPPER>
 __global__ void __launch_bounds__(256) k_gemm_nn(const F* __restrict__ A, long long lda,
                                                   const F* __restrict__ Q, int ldq,
@@ -263,7 +269,6 @@ __global__ void __launch_bounds__(256) k_gemm_nn(const F* __restrict__ A, long l
   MacAcc<Cm> acc[4][U];
   const int kend = UPPER ? min(K, j0 + BN) : K;
   for (int k0 = 0; k0 < kend; k0 += GK) {
-    const int v0 = UPPER ? max(0, (k0 - j0) / 16) : 0;  // first column group that k0 reaches
     for (int idx = tid; idx < GK * BM; idx += 256) {
       int rr = idx % BM, kk = idx / BM;
       long long r = r0 + rr;
@@ -284,11 +289,9 @@ __global__ void __launch_bounds__(256) k_gemm_nn(const F* __restrict__ A, long l
 #pragma unroll
       for (int v = 0; v < U; ++v) b[v] = Qs[kk][ty + 16 * v];
 #pragma unroll
-      for (int v = 0; v < U; ++v) {
-        if (UPPER && v < v0) continue;
+      for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u][v].add_prod(a[u], b[v]);
-      }
+        for (int v = 0; v < U; ++v) acc[u][v].add_prod(a[u], b[v]);
     }
     __syncthreads();
   }
@@ -310,7 +313,8 @@ __global__ void __launch_bounds__(256) k_gemm_nn(const F* __restrict__ A, long l
 
 // The double-float rotation on packed FP32 instructions: a thread owns 4 consecutive rows (two
 // operand pairs as they lie in shared memory) x U columns; the factor's values are stored twice
-// over, so that one 16-byte load gives both broadcast pairs. UPPER as in k_gemm_nn.
+// over, so that one 16-byte load gives both broadcast pairs. The sums round as in k_gemm_nn. UPPER:
+// a step of 16 rows k of Q meets only the column groups of 16 that reach it (15 of 25 at 80 columns).
 template <int U, int V0>
 __device__ __forceinline__ void nn_df_step(const float* Ah, const float* Al, const float4* Qs,
                                            int tx, int ty, df64acc2 (&acc)[2][U]) {
@@ -390,19 +394,30 @@ static cudaError_t gemm_nn_impl(const F* A, long long lda, const F* Q, int ldq, 
                                 cudaStream_t stream, bool upper) {
   const int u = tile_u(n);
   dim3 grid((unsigned)((d + 63) / 64), (n + 16 * u - 1) / (16 * u));
-#define CS_NN_CASE(UV)                                                                       \
-  case UV:                                                                                   \
-    if constexpr (std::is_same<Cm, df64>::value) {                                           \
-      if (upper)                                                                             \
-        k_gemm_nn_df<UV, true><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, C, ldc);   \
-      else                                                                                   \
-        k_gemm_nn_df<UV, false><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, C, ldc);  \
-    } else if (upper)                                                                               \
+  // Double-float: the packed form from three column groups on, for a triangular factor, whose zeros
+  // it skips (97 columns, d = 6936: 78 -> 69 us), or where the grid has two waves of two CTAs per
+  // SM (300 columns, d = 46128: 2162 -> 1898; at d = 6936 326 -> 340). With one or two groups a
+  // thread's operands cost more than the sums (10 -> 14 us at 5 columns), with six the full form
+  // has too many registers (81 columns: 210 -> 223).
+  const bool packed = std::is_same<Cm, df64>::value && u >= 3 &&
+                      (upper || (u <= 5 && (long long)grid.x * grid.y >= 608));
+#define CS_NN_CASE(UV)                                                                        \
+  case UV:                                                                                    \
+    if constexpr (std::is_same<Cm, df64>::value && UV >= 3) {                                 \
+      if (packed) {                                                                           \
+        if (upper)                                                                            \
+          k_gemm_nn_df<UV, true><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, C, ldc);  \
+        else if constexpr (UV <= 5)                                                           \
+          k_gemm_nn_df<UV, false><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, C, ldc); \
+        break;                                                                                \
+      }                                                                                       \
+    }                                                                                         \
+    if (upper)                                                                                \
       k_gemm_nn<F, Cm, UV, true><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, \
-                                                           (F)beta, C, ldc);                 \
-    else                                                                                     \
+                                                           (F)beta, C, ldc);                  \
+    else                                                                                      \
       k_gemm_nn<F, Cm, UV, false><<<grid, 256, 0, stream>>>(A, lda, Q, ldq, d, k, n, (F)alpha, \
-                                                            (F)beta, C, ldc);                \
+                                                            (F)beta, C, ldc);                 \
     break;
   switch (u) {
     CS_NN_CASE(1)
