@@ -30,8 +30,6 @@ struct Layout {
 };
 
 constexpr int kMaxLanczos = 64;
-// largest block whose eigensolve starts with the one-CTA FP32 stage (launch_sym_eig)
-constexpr int kOneCtaEig = 112;
 // largest degree of the residual-form filter (its weight table is sized for it)
 constexpr int kMaxRitzDegree = 64;
 
@@ -535,11 +533,11 @@ cs_status rr_core(cs_ctx* c, int n_s, double* X, long long ld, double* theta, do
   double* Q = Hs + (size_t)n_s * n_s;
   double* jw = Q + (size_t)n_s * n_s;
   cs_status r;
-  // Above kOneCtaEig states the eigensolver works in FP64 throughout and the signs of its vectors
+  // Where the one-CTA stage has no room (above 112 states) the eigensolver works in FP64 throughout and the signs of its vectors
   // follow the last bits of the projected matrix, so there the H X keeps the FMA kernels'
   // rounding: X and HX_out would come back with other signs for the same block (880 states:
   // 256 ms with the slice products, 494 without).
-  const bool fma = n_s > kOneCtaEig;
+  const bool fma = !sym_eig_one_cta(n_s);
   if (c->rr_prec == CS_FP64) {
     r = hx_core<double>(c, n_s, X, ld, HX, H.d, EP_APPLY, 0, 0, 0, nullptr, work, st, false,
                         nullptr, nullptr, nullptr, false, fma);

@@ -158,6 +158,9 @@ cudaError_t launch_cholqr_factor(const double* M, int n, double* U, double* work
                                  cudaStream_t stream);
 // A (n x n) <- (A + A^T) / 2
 cudaError_t launch_symmetrize(double* A, int n, cudaStream_t stream);
+// whether a block of n states fits the eigensolver's one-CTA FP32 stage (n <= 112); above, its
+// first stage is FP64 and device-wide
+bool sym_eig_one_cta(int n);
 // Symmetric eigensolve of sym(A) (n x n, lda = n): theta ascending, V (n x n) columns. An FP32
 // solve (Householder tridiagonalisation, then bisection with inverse iteration, or QL where the
 // bisection tiles do not fit in shared memory), Newton-Schulz re-orthonormalisation and

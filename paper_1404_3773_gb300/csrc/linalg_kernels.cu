@@ -1831,6 +1831,11 @@ cudaError_t launch_symmetrize(double* A, int n, cudaStream_t stream) {
   return cudaGetLastError();
 }
 
+static size_t one_cta_eig_smem(int n) {
+  return (4 * (size_t)n * n + 7 * (size_t)n) * sizeof(float);
+}
+bool sym_eig_one_cta(int n) { return one_cta_eig_smem(n) <= 200 * 1024; }
+
 cudaError_t launch_sym_eig(const double* A, int n, double* theta, double* V, double* work,
                               int* status, cudaStream_t stream, void* oz, size_t oz_bytes,
                               int* oz_err) {
@@ -1854,8 +1859,8 @@ cudaError_t launch_sym_eig(const double* A, int n, double* theta, double* V, dou
   }
   // 1. FP32 eigendecomposition of sym(A) -> V0 (FP64 copy of the FP32 vectors)
   cudaError_t e;
-  const size_t smem_b = (4 * n2 + 7 * (size_t)n) * sizeof(float);
-  if (smem_b <= 200 * 1024) {
+  const size_t smem_b = one_cta_eig_smem(n);
+  if (sym_eig_one_cta(n)) {
     // bisection + inverse iteration on the tridiagonal (parallel over eigenvalues)
     e = cudaFuncSetAttribute(k_sym_eig<float, true, true>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b);
