@@ -490,7 +490,7 @@ cudaError_t dense_rotate(const cs_ctx* c, const double* A, long long lda, const 
   if (c->dense_prec == CS_FP64_SLICED)
     return launch_oz_rotate(A, lda, Q, ldq, d, k, n, C, ldc, oz, c->dev_err, st, upper);
   return c->dense_prec == CS_DF64
-             ? launch_gemm_nn_df(A, lda, Q, ldq, d, k, n, 1.0, 0.0, C, ldc, st, upper)
+             ? launch_gemm_nn_df(A, lda, Q, ldq, d, k, n, C, ldc, st, upper)
              : launch_gemm_nn<double>(A, lda, Q, ldq, d, k, n, 1.0, 0.0, C, ldc, st, upper);
 }
 

@@ -142,13 +142,13 @@ template <typename F>
 cudaError_t launch_gemm_nn(const F* A, long long lda, const F* Q, int ldq, long long d, int k,
                            int n, double alpha, double beta, F* C, long long ldc,
                            cudaStream_t stream, bool upper = false);
-// the same two products on FP64 arrays with double-float arithmetic (FP32 pipe); alpha 1, beta 0
+// A^T B, and A Q alone, on FP64 arrays with double-float arithmetic (FP32 pipe)
 cudaError_t launch_gram_df(const double* A, long long lda, const double* B, long long ldb,
                            long long d, int na, int nb, double* C, int ldc, double* partial,
                            cudaStream_t stream);
 cudaError_t launch_gemm_nn_df(const double* A, long long lda, const double* Q, int ldq,
-                              long long d, int k, int n, double alpha, double beta, double* C,
-                              long long ldc, cudaStream_t stream, bool upper = false);
+                              long long d, int k, int n, double* C, long long ldc,
+                              cudaStream_t stream, bool upper = false);
 // y[p + s ld] *= h[p] for p < n_p, s < S
 template <typename F>
 cudaError_t launch_scale_rows(F* y, int n_p, int S, int ld, const F* h, cudaStream_t stream);

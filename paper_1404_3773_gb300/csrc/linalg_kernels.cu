@@ -440,10 +440,9 @@ cudaError_t launch_gemm_nn(const F* A, long long lda, const F* Q, int ldq, long 
 }
 
 cudaError_t launch_gemm_nn_df(const double* A, long long lda, const double* Q, int ldq,
-                              long long d, int k, int n, double alpha, double beta, double* C,
-                              long long ldc, cudaStream_t stream, bool upper) {
-  if (alpha != 1.0 || beta != 0.0) return cudaErrorInvalidValue;
-  return gemm_nn_impl<double, df64>(A, lda, Q, ldq, d, k, n, alpha, beta, C, ldc, stream, upper);
+                              long long d, int k, int n, double* C, long long ldc,
+                              cudaStream_t stream, bool upper) {
+  return gemm_nn_impl<double, df64>(A, lda, Q, ldq, d, k, n, 1.0, 0.0, C, ldc, stream, upper);
 }
 
 template cudaError_t launch_gram<double>(const double*, long long, const double*, long long,
