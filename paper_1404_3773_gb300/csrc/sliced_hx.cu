@@ -41,6 +41,7 @@
 #include <vector>
 
 #include "cs_internal.h"
+#include "hx_device.cuh"
 #include "hx_kernels.cuh"
 #include "image_ring.cuh"
 #include "ozaki_split.cuh"
@@ -657,29 +658,13 @@ __global__ void __launch_bounds__(kSlThreads, sl_ctas(OP, NB)) k_sl(SlArgs a) {
       }
       if constexpr (OP == OP_R2) {
         if (ok && w.live) {
-          const Epilogue<double>& ep = a.ep;
 #pragma unroll
           for (int c = 0; c < HC; ++c) {
             const int n = NB * st + half * HC + c;
             if (n >= a.N) continue;
             const double z = to_f64(acc[c], rowsc + __ldg(a.fexp + w.l * a.N + n) - 54);
             const size_t al = (size_t)(w.l * w.l + w.mi) * a.N + n;
-            const size_t o = al + (size_t)w.s * ep.ld_out;
-            if (ep.mode == EP_PLAIN) {
-              ep.out[o] = z;
-              continue;
-            }
-            const double x = ep.X[al + (size_t)w.s * ep.ld];
-            double hx = ep.half_lambda[al] * x + z;
-            if (ep.kb) hx += ep.kb[al + (size_t)w.s * ep.kb_ld];
-            if (ep.src) hx += ep.src_w[w.s] * ep.src[al + (size_t)w.s * ep.src_ld];
-            if (ep.mode == EP_APPLY) {
-              ep.out[o] = hx;
-            } else {
-              double y = ep.cA * (hx - ep.cshift * x);
-              if (ep.Yprev) y -= ep.cB * ep.Yprev[o];
-              ep.out[o] = y;
-            }
+            radial_epilogue(a.ep, al, w.s, z);
           }
         }
       }
