@@ -70,7 +70,8 @@ typedef enum {
   CS_FP64 = 0,       /* FP64 storage and accuracy: FP64 arithmetic, or, for blocks from 4096
                         grid rows x states (N_r N_theta n_s), exact products of 8-bit integer
                         slices on the tensor cores with 64-bit integer sums between them
-                        (agreement with the FP64 arithmetic to a few units of 2^-53)      */
+                        (agreement with the FP64 arithmetic to a few units of 2^-53;
+                        Rayleigh-Ritz of more than 112 states keeps FP64 arithmetic)      */
   CS_FP32 = 1,       /* FP32 storage and arithmetic (FP32 FMA pipe)                      */
   CS_MIXED_BF16 = 2  /* FP32 storage; the per-l radial contractions on the tensor cores
                         (tcgen05) with operands split into two BF16 terms (hi + lo, three
@@ -84,7 +85,8 @@ typedef enum {
                         transformations). On a GPU whose FP64 pipe runs at 1/64 of the FP32
                         rate this is faster than FP64 arithmetic at relative errors near 1e-14.
                         Blocks with N_r N_theta n_s (lmax+1)^2 >= 14e6 take CS_FP64's slice
-                        products instead. With projectors it is available for cs_apply_H and the
+                        products instead (not in Rayleigh-Ritz of more than 112 states). With
+                        projectors it is available for cs_apply_H and the
                         Rayleigh-Ritz apply only, and only with CS_FP64_SLICED dense
                         products (the projector term is then formed as exact slice products
                         and added in double-float); CS_ERR_STATE otherwise.               */,

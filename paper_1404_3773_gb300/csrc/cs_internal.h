@@ -106,8 +106,7 @@ namespace cs {
 // (sliced_hx.cu), by the number of grid rows x states.
 // FP64: they are faster at every size measured (lmax 6 .. 60, 1 .. 130 states): 0.074 against
 // 0.092 ms at 3456 rows, where launches dominate, 0.084 against 0.134 at 5120, 1.50 against 7.13
-// at 460800 (lmax 30, 80 states). Below 4096 rows, with little to gain, the kernels that
-// cs_apply_H_noalloc runs stay.
+// at 460800 (lmax 30, 80 states). Below 4096 rows, with little to gain, the FMA kernels stay.
 // Double-float: its kernels cost less per row at small lmax. rows L^2 = 14M is where the two
 // meet: 0.130 / 0.122 ms at 7.4M (lmax 16, 16 states), 0.177 / 0.181 at 15M (lmax 23, 8),
 // 0.168 / 0.193 at 15M (lmax 16, 32), 0.254 / 0.336 at 44M (lmax 30, 8).

@@ -25,7 +25,7 @@
 //
 // The kernels are bound by the instructions of splitting (about 40 per value with its load) and
 // joining (about 25): 0.75 G warp instructions for 80 states at lmax 30, issued at 35 % (radial) to
-// 60 % of the peak rate; the tensor cores are idle most of the time. That H.X takes 1.51 ms against
+// 60 % of the peak rate; the tensor cores are idle most of the time. That H.X takes 1.48 ms against
 // 7.13 on the FP64 pipe (whose peak would need 2.9 ms) and 2.41 in double-float. Two to four CTAs
 // of 256 threads run per SM, so one CTA's loads and drains cover the others' waits. A thread owns the same
 // operand row when it loads and when it drains, so its row's scale never leaves its registers.
